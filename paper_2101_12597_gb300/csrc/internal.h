@@ -281,6 +281,14 @@ struct KGeom {
   const double *kfrac;  // [nk][3] k-points in fractional reciprocal coordinates (device)
 };
 
+// Workspace of the full-A path's tensor-core products (ozgemm.cu): base-256
+// digits of both operands for `group` n x n matrices at a time (n = 0: none).
+struct OzWork {
+  int n = 0, group = 0, sms = 0;
+  uint8_t *a = nullptr, *b = nullptr;
+  int *rexp = nullptr, *cexp = nullptr;
+};
+
 }  // namespace etdm
 
 struct etdm_handle {
@@ -309,6 +317,7 @@ struct etdm_handle {
   double2 *d_kX1 = nullptr, *d_kX2 = nullptr;
   double *d_kDR = nullptr, *d_kVR = nullptr;  // [nR][M][M]
   void *d_kwork = nullptr;      // eigensolver workspace
+  etdm::OzWork oz{};            // tensor-core products (large M)
   bool kref_set = false;        // reference given by etdm_set_reference
   int kexpm = 0;                // ETDM_EXPM_EIG (Eq. 35, Eq. 39) or ETDM_EXPM_SS (Eq. 38, Eq. 42)
   int tri_method = 1;           // tridiagonal eigenpairs of iA(k): 1 bisection + inverse iteration, 0 QL

@@ -34,6 +34,14 @@ void check_device_status(etdm_handle *h, cudaStream_t s, const char *where) {
   throw Fail{code, std::string(where) + ": S(k) not positive definite or a non-finite value"};
 }
 
+// C = alpha op(A) op(B) + beta C for every k-point: on the tensor cores when
+// the handle has their workspace (M >= kOzMin), else FP64 FMA
+cudaError_t prod_k(etdm_handle *h, const double2 *A, int opa, const double2 *B, int opb, double2 *C,
+                   cudaStream_t s, double alpha = 1.0, double beta = 0.0) {
+  if (h->oz.n == h->M) return launch_oz_zgemm(h->oz, A, opa, B, opb, C, h->nk, alpha, beta, h->d_flags, s);
+  return zgemm_sq(A, opa, B, opb, C, h->M, h->nk, s, alpha, beta);
+}
+
 }  // namespace
 
 void init_kpoints(etdm_handle *h, const etdm_system *sys) {
@@ -83,6 +91,8 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
     h->d_knorm = dalloc<unsigned long long>(h, 1);
     h->d_kfro = dalloc<double>(h, 2 * k_fro2_parts());
   }
+
+  if (M >= kOzMin) oz_alloc(h, M, nk);
 
   // S(k), T(k); h_core(k) = T(k) + V_ext(k)
   CUDA_TRY(k_overlap_kinetic(h, s));
@@ -138,8 +148,8 @@ void expm_ss_k(etdm_handle *h, const double *a, double2 *U, cudaStream_t s) {
   int sq = 0;
   while (ldexp(1.0, sq) < nrm) ++sq;
   if (sq > 0) CUDA_TRY(k_build_iA(a, nk, M, h->d_kB, s, 0, ldexp(1.0, -sq)));
-  CUDA_TRY(zgemm_sq(h->d_kB, 0, h->d_kB, 0, h->d_kB2, M, nk, s));   // B^2
-  CUDA_TRY(zgemm_sq(h->d_kB2, 0, h->d_kB, 0, h->d_kB3, M, nk, s));  // B^3
+  CUDA_TRY(prod_k(h, h->d_kB, 0, h->d_kB, 0, h->d_kB2, s));   // B^2
+  CUDA_TRY(prod_k(h, h->d_kB2, 0, h->d_kB, 0, h->d_kB3, s));  // B^3
   double c[19];
   c[0] = 1.0;
   for (int j = 1; j <= 18; ++j) c[j] = c[j - 1] / j;
@@ -147,11 +157,11 @@ void expm_ss_k(etdm_handle *h, const double *a, double2 *U, cudaStream_t s) {
   CUDA_TRY(k_poly(Y, h->d_kB, h->d_kB2, c[18], 0.0, 0.0, nk, M, s));  // c18 I
   for (int i = 5; i >= 0; --i) {  // Y <- q_i + B^3 Y
     CUDA_TRY(k_poly(Yn, h->d_kB, h->d_kB2, c[3 * i], c[3 * i + 1], c[3 * i + 2], nk, M, s));
-    CUDA_TRY(zgemm_sq(h->d_kB3, 0, Y, 0, Yn, M, nk, s, 1.0, 1.0));
+    CUDA_TRY(prod_k(h, h->d_kB3, 0, Y, 0, Yn, s, 1.0, 1.0));
     std::swap(Y, Yn);
   }
   for (int j = 0; j < sq; ++j) {  // square s times
-    CUDA_TRY(zgemm_sq(Y, 0, Y, 0, Yn, M, nk, s));
+    CUDA_TRY(prod_k(h, Y, 0, Y, 0, Yn, s));
     std::swap(Y, Yn);
   }
   CUDA_TRY(cudaMemcpyAsync(U, Y, (size_t)nk * M * M * 16, cudaMemcpyDeviceToDevice, s));
@@ -200,7 +210,7 @@ void refresh_reference_k(etdm_handle *h, cudaStream_t s) {
   const int M = h->M, nk = h->nk;
   CUDA_TRY(cudaMemsetAsync(h->d_a, 0, h->nvar * 8, s));
   evaluate_k(h, h->d_a, h->d_E, h->d_g, s);
-  CUDA_TRY(zgemm_sq(h->d_kH, 0, h->d_kC0, 0, h->d_kX1, M, nk, s));
+  CUDA_TRY(prod_k(h, h->d_kH, 0, h->d_kC0, 0, h->d_kX1, s));
   CUDA_TRY(k_diag(h->d_kC0, h->d_kX1, h->d_eps, nk, M, s));
   CUDA_TRY(k_precond_parts(h->d_eps, h->d_kf, h->d_kw, nk, M, h->gamma, h->d_kpden, h->d_kpw, s));
 }
@@ -208,7 +218,7 @@ void refresh_reference_k(etdm_handle *h, cudaStream_t s) {
 void reference_update_k(etdm_handle *h, double *a, cudaStream_t s) {
   const int M = h->M, nk = h->nk;
   expm_ss_k(h, a, h->d_kW, s);
-  CUDA_TRY(zgemm_sq(h->d_kC0, 0, h->d_kW, 0, h->d_kX1, M, nk, s));
+  CUDA_TRY(prod_k(h, h->d_kC0, 0, h->d_kW, 0, h->d_kX1, s));
   CUDA_TRY(cudaMemcpyAsync(h->d_kC0, h->d_kX1, (size_t)nk * M * M * 16, cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(cudaMemsetAsync(a, 0, h->nvar * 8, s));
   refresh_reference_k(h, s);
@@ -220,8 +230,8 @@ void commutator_norms_k(etdm_handle *h, const double *a, const double *g, double
   const long KM = (long)nk * M * M;
   CUDA_TRY(k_build_iA(a, nk, M, h->d_kB, s, 0, 1.0));   // A
   CUDA_TRY(k_from_grad(g, h->d_kB2, nk, M, s));         // L
-  CUDA_TRY(zgemm_sq(h->d_kB, 0, h->d_kB2, 0, h->d_kB3, M, nk, s));                  // A L
-  CUDA_TRY(zgemm_sq(h->d_kB2, 0, h->d_kB, 0, h->d_kB3, M, nk, s, -1.0, 1.0));       // - L A
+  CUDA_TRY(prod_k(h, h->d_kB, 0, h->d_kB2, 0, h->d_kB3, s));                  // A L
+  CUDA_TRY(prod_k(h, h->d_kB2, 0, h->d_kB, 0, h->d_kB3, s, -1.0, 1.0));       // - L A
   CUDA_TRY(k_fro2(h->d_kB2, KM, h->d_kfro, s));
   CUDA_TRY(k_fro2(h->d_kB3, KM, h->d_kfro + k_fro2_parts(), s));
   std::vector<double> part(2 * k_fro2_parts());
@@ -255,14 +265,14 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   }
   StageTimer tf(h, s, ETDM_STAGE_DENSE_FWD);
   if (ss) {
-    CUDA_TRY(zgemm_sq(h->d_kC0, 0, h->d_kW, 0, h->d_kO, M, nk, s));    // O = C0 U
+    CUDA_TRY(prod_k(h, h->d_kC0, 0, h->d_kW, 0, h->d_kO, s));    // O = C0 U
   } else {
     CUDA_TRY(k_colscale(h->d_kW, h->d_komega, h->d_kX1, nk, M, 2, h->d_flags, s));
-    CUDA_TRY(zgemm_sq(h->d_kX1, 0, h->d_kW, 1, h->d_kX2, M, nk, s));    // U
-    CUDA_TRY(zgemm_sq(h->d_kC0, 0, h->d_kX2, 0, h->d_kO, M, nk, s));    // O = C0 U
+    CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kW, 1, h->d_kX2, s));    // U
+    CUDA_TRY(prod_k(h, h->d_kC0, 0, h->d_kX2, 0, h->d_kO, s));    // O = C0 U
   }
   CUDA_TRY(k_colscale(h->d_kO, h->d_kf, h->d_kX1, nk, M, 0, h->d_flags, s));
-  CUDA_TRY(zgemm_sq(h->d_kX1, 0, h->d_kO, 1, h->d_kD, M, nk, s));     // D = O f O^dagger
+  CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kO, 1, h->d_kD, s));     // D = O f O^dagger
   CUDA_TRY(k_dr(G, h->d_kD, h->d_kDR, s));
   tf.done();
   // density, potential, energy
@@ -295,8 +305,8 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   tv.done();
   StageTimer tg(h, s, ETDM_STAGE_DENSE_REV);
   CUDA_TRY(k_hamiltonian(G, h->d_kT, h->d_kVR, h->d_kH, s));
-  CUDA_TRY(zgemm_sq(h->d_kH, 0, h->d_kO, 0, h->d_kX1, M, nk, s));     // H O
-  CUDA_TRY(zgemm_sq(h->d_kO, 1, h->d_kX1, 0, h->d_kX2, M, nk, s));    // O^dagger H O
+  CUDA_TRY(prod_k(h, h->d_kH, 0, h->d_kO, 0, h->d_kX1, s));     // H O
+  CUDA_TRY(prod_k(h, h->d_kO, 1, h->d_kX1, 0, h->d_kX2, s));    // O^dagger H O
   CUDA_TRY(k_commutator(h->d_kX2, h->d_kf, nk, M, s));                // L
   if (h->sic) CUDA_TRY(k_sic_L(h->d_kX2, h->d_sicS, h->d_kf, M, s));   // orbital potentials
   if (ss) {  // Eq. 42: G ~ L^T
@@ -305,11 +315,11 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
     h->launches += 5;
     return;
   }
-  CUDA_TRY(zgemm_sq(h->d_kX2, 0, h->d_kW, 0, h->d_kX1, M, nk, s));    // L W
-  CUDA_TRY(zgemm_sq(h->d_kW, 1, h->d_kX1, 0, h->d_kX2, M, nk, s));    // W^dagger L W
+  CUDA_TRY(prod_k(h, h->d_kX2, 0, h->d_kW, 0, h->d_kX1, s));    // L W
+  CUDA_TRY(prod_k(h, h->d_kW, 1, h->d_kX1, 0, h->d_kX2, s));    // W^dagger L W
   CUDA_TRY(k_dtilde(h->d_kX2, h->d_komega, nk, M, s));
-  CUDA_TRY(zgemm_sq(h->d_kW, 0, h->d_kX2, 0, h->d_kX1, M, nk, s));
-  CUDA_TRY(zgemm_sq(h->d_kX1, 0, h->d_kW, 1, h->d_kX2, M, nk, s));    // G^T
+  CUDA_TRY(prod_k(h, h->d_kW, 0, h->d_kX2, 0, h->d_kX1, s));
+  CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kW, 1, h->d_kX2, s));    // G^T
   CUDA_TRY(k_grad_vars(h->d_kX2, g, nk, M, s));
   tg.done();
   h->launches += 11;

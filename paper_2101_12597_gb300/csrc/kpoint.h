@@ -24,6 +24,13 @@ cudaError_t launch_zgemm(const ZgemmArgs &g, int batch, cudaStream_t s);
 cudaError_t zgemm_sq(const double2 *A, int opa, const double2 *B, int opb, double2 *C, int n,
                      int batch, cudaStream_t s, double alpha = 1.0, double beta = 0.0);
 
+// the same products on the tensor cores, as accurate as FP64 arithmetic (ozgemm.cu)
+constexpr int kOzMin = 64;  // smallest matrices that take them
+void oz_alloc(etdm_handle *h, int n, int batch);
+cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const double2 *B, int opb,
+                            double2 *C, int batch, double alpha, double beta, int *flags,
+                            cudaStream_t s);
+
 // Hermitian eigensolver: A (destroyed) = V diag(w) V^dagger, w ascending.
 size_t heev_work_bytes(int n, int batch);
 // method 0: implicit QL on the tridiagonal (robust for any spectrum; used at
