@@ -370,7 +370,7 @@ const char *etdm_last_error(const etdm_handle *h);
  * that only hand out pre-registered buffers, drivers that forbid cudaMalloc
  * after start-up).  It computes p = -H g with the same two-loop recursion as
  * etdm_lbfgs_step, from a pair history the caller keeps, and allocates
- * nothing: its reduction scratch is a fixed 2.3 KB file-scope device array.
+ * nothing: its reduction scratch is a fixed 8.3 KB file-scope device array.
  *   g_dev  [n]      gradient
  *   s_dev  [m*n]    steps s_i = a_(i+1) - a_i, oldest (i = 0) to newest
  *   y_dev  [m*n]    gradient changes y_i; every pair needs y_i . s_i > 0
