@@ -279,6 +279,7 @@ struct KGeom {
   int Rm[3];
   int nR;
   const double *kfrac;  // [nk][3] k-points in fractional reciprocal coordinates (device)
+  const double2 *phase; // [nR][nk] exp(2 pi i k.R) (device)
 };
 
 // Workspace of the full-A path's tensor-core products (ozgemm.cu): base-256

@@ -35,7 +35,7 @@ void check_device_status(etdm_handle *h, cudaStream_t s, const char *where) {
 }
 
 // C = alpha op(A) op(B) + beta C for every k-point: on the tensor cores when
-// the handle has their workspace (M >= kOzMin), else FP64 FMA
+// the handle has their workspace (oz_takes), else FP64 FMA
 cudaError_t prod_k(etdm_handle *h, const double2 *A, int opa, const double2 *B, int opb, double2 *C,
                    cudaStream_t s, double alpha = 1.0, double beta = 0.0) {
   if (h->oz.n == h->M) return launch_oz_zgemm(h->oz, A, opa, B, opb, C, h->nk, alpha, beta, h->d_flags, s);
@@ -61,6 +61,9 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
   h->d_kfrac = dupload(h, h->h_kfrac.data(), 3 * (size_t)nk);
   h->d_kw = dupload(h, h->h_kw.data(), (size_t)nk);
   G.kfrac = h->d_kfrac;
+  double2 *phase = dalloc<double2>(h, (size_t)G.nR * nk);
+  CUDA_TRY(k_phases(G, phase, s));
+  G.phase = phase;
   h->N = sys->n_electrons / 2;
   h->V = M - h->N;
   h->nvar = KM;
@@ -92,7 +95,7 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
     h->d_kfro = dalloc<double>(h, 2 * k_fro2_parts());
   }
 
-  if (M >= kOzMin) oz_alloc(h, M, nk);
+  if (oz_takes(M, nk)) oz_alloc(h, M, nk);
 
   // S(k), T(k); h_core(k) = T(k) + V_ext(k)
   CUDA_TRY(k_overlap_kinetic(h, s));

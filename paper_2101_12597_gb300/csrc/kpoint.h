@@ -25,7 +25,11 @@ cudaError_t zgemm_sq(const double2 *A, int opa, const double2 *B, int opb, doubl
                      int batch, cudaStream_t s, double alpha = 1.0, double beta = 0.0);
 
 // the same products on the tensor cores, as accurate as FP64 arithmetic (ozgemm.cu)
-constexpr int kOzMin = 64;  // smallest matrices that take them
+// Which products take them: 64 rows at least (half a tile of 128 rows is
+// padding there) and n^3 x batch from which the FP64 kernel's 4 n^3 batch /
+// 2.6e11 s pass the 25 us or so that the digits and one tile's K loop take at
+// least (n = 129, 3 matrices: 52 us against 100; n = 64, 3: 32 against 12)
+inline bool oz_takes(int n, int batch) { return n >= 64 && (double)n * n * n * batch >= 3e6; }
 void oz_alloc(etdm_handle *h, int n, int batch);
 cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const double2 *B, int opb,
                             double2 *C, int batch, double alpha, double beta, int *flags,
@@ -57,6 +61,7 @@ cudaError_t k_fro2(const double2 *X, long n, double *part, cudaStream_t s);
 cudaError_t k_colscale(const double2 *Y, const double *x, double2 *X, int nk, int M, int mode,
                        int *flags, cudaStream_t s);
 cudaError_t k_hermitize(double2 *X, int nk, int M, cudaStream_t s);
+cudaError_t k_phases(const KGeom &G, double2 *phase, cudaStream_t s);  // fills G.phase's table (set-up)
 cudaError_t k_dr(const KGeom &G, const double2 *D, double *DR, cudaStream_t s);
 cudaError_t k_hamiltonian(const KGeom &G, const double2 *T, const double *VR, double2 *H,
                           cudaStream_t s);

@@ -1,7 +1,8 @@
 """The full-A path's complex products at the sizes where their kernels can go
-wrong, through E and the gradient against the k-point oracle: the smallest
-matrices on the tensor cores (64), a K tail and a partial column tile (72), a
-second block of 128 rows (135, one k-point), with exp(A) by both routes."""
+wrong, through E and the gradient against the k-point oracle: FP64 tiles with
+a remainder and one k-point (20), the largest on the FP64 kernel (64), tensor
+cores with a K tail and a partial column tile (80), a second block of 128 rows
+(144); with exp(A) by both routes."""
 import numpy as np
 import pytest
 
@@ -11,9 +12,10 @@ from oracle.etdm_kpoints import BlochOracle
 pytestmark = pytest.mark.gpu
 
 SYSTEMS = {
+    20: dict(cells=(2, 1, 2), n_exp=5, grid=(16, 15, 14), kmesh=1),
     64: dict(cells=(2, 2, 2), n_exp=8, grid=(16, 15, 14), kmesh=2),
-    72: dict(cells=(3, 2, 3), n_exp=4, grid=(18, 14, 16), kmesh=2),
-    135: dict(cells=(3, 3, 3), n_exp=5, grid=(20, 18, 18), kmesh=1),
+    80: dict(cells=(2, 5, 2), n_exp=4, grid=(14, 24, 15), kmesh=2),
+    144: dict(cells=(3, 3, 4), n_exp=4, grid=(20, 18, 24), kmesh=1),
 }
 
 
