@@ -15,7 +15,7 @@ SYSTEMS = {
     20: dict(cells=(2, 1, 2), n_exp=5, grid=(16, 15, 14), kmesh=1),
     64: dict(cells=(2, 2, 2), n_exp=8, grid=(16, 15, 14), kmesh=2),
     80: dict(cells=(2, 5, 2), n_exp=4, grid=(14, 24, 15), kmesh=2),
-    144: dict(cells=(3, 3, 4), n_exp=4, grid=(20, 18, 24), kmesh=1),
+    144: dict(cells=(3, 3, 4), n_exp=4, grid=(20, 18, 24), kmesh=2),
 }
 
 
