@@ -207,10 +207,19 @@ __device__ __noinline__ void phase_tile(const Phase &ph, int tile, R (*As)[2][BM
       const bool more = it + 1 < nit;
       if (more) load(KG * (it + 1) + grp);
       if (it < nit) {
+        const int kn = ph.k - (KG * it + grp) * BK;
+        if (kn >= BK) {
 #pragma unroll
-        for (int kk = 0; kk < BK; kk += 4) {
+          for (int kk = 0; kk < BK; kk += 4) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) mac.step(u, As[grp][buf][ty][kk + u], Bs[grp][buf][kk + u][tx]);
+            for (int u = 0; u < 4; ++u) mac.step(u, As[grp][buf][ty][kk + u], Bs[grp][buf][kk + u][tx]);
+          }
+        } else {  // K's tail, in whole steps of four (zeros beyond K)
+#pragma unroll 1
+          for (int kk = 0; kk < kn; kk += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) mac.step(u, As[grp][buf][ty][kk + u], Bs[grp][buf][kk + u][tx]);
+          }
         }
       }
       if (more) store(buf ^ 1);
@@ -222,10 +231,9 @@ __device__ __noinline__ void phase_tile(const Phase &ph, int tile, R (*As)[2][BM
   __syncthreads();
   if (grp == 0 && i < ph.m && j < ph.n) {
     R v = acc;
-#pragma unroll
-    for (int q = 0; q < KG - 1; ++q) v = X::add(v, part[q][tid]);
+    for (int q = 0; q < min(KG, nch) - 1; ++q) v = X::add(v, part[q][tid]);
     for (int q = 0; q < ph.nc; ++q) v = X::fma(ph.beta[q], X::ld(ph.C[q], (long)i * ph.ldc[q] + j), v);
-    if (i == j) v = X::add(v, X::from(ph.diag));
+    if (i == j && ph.diag != 0.0) v = X::add(v, X::from(ph.diag));
     const long o = (long)i * ph.ldo + j;
     if (ph.out64) static_cast<double *>(ph.out)[o] = X::dbl(v);
     else X::st(ph.out, o, v);
@@ -235,6 +243,61 @@ __device__ __noinline__ void phase_tile(const Phase &ph, int tile, R (*As)[2][BM
     }
   }
   __syncthreads();
+}
+
+// A small phase on one block (K of two chunks at most): a thread per output,
+// operands straight from L1, the same sums as phase_tile makes (four
+// multiply-add chains per chunk, chunks added in order), without its staging,
+// padding and four block barriers; a phase of a 16 x 4 system took 4 to 5 us in
+// tiles.
+constexpr int kDirectK = 2 * BK, kDirectOut = 2 * NT;
+__device__ __forceinline__ bool use_direct(const Phase &ph, int nb) {
+  return nb == 1 && ph.k <= kDirectK && ph.m * ph.n <= kDirectOut;
+}
+template <class R>
+__device__ __noinline__ void phase_direct(const Phase &ph, double *sq) {
+  using X = Num<R>;
+  const int m = ph.m, n = ph.n, K = ph.k;
+  for (int e = threadIdx.x; e < m * n; e += NT) {
+    const int i = e / n, j = e % n;
+    R acc[2] = {X::zero(), X::zero()};
+    for (int q = 0; q < ph.np; ++q) {
+      const Prod &P = ph.p[q];
+      const double alpha = P.alpha;
+      if (alpha == 0.0) continue;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int k0 = c * BK, k1 = min(K, k0 + BK);
+        if (k0 >= K) break;
+        Mac<R> mac;
+#pragma unroll 2
+        for (int k = k0; k < k1; k += 4) {
+          R a[4], bb[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            a[u] = bb[u] = X::zero();
+            if (k + u < k1) {
+              a[u] = opA<R>(P, i, k + u);
+              bb[u] = opB<R>(P, k + u, j);
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) mac.step(u, a[u], bb[u]);
+        }
+        acc[c] = X::fma(alpha, mac.total(), acc[c]);
+      }
+    }
+    R v = K > BK ? X::add(acc[0], acc[1]) : acc[0];
+    for (int q = 0; q < ph.nc; ++q) v = X::fma(ph.beta[q], X::ld(ph.C[q], (long)i * ph.ldc[q] + j), v);
+    if (i == j && ph.diag != 0.0) v = X::add(v, X::from(ph.diag));
+    const long o = (long)i * ph.ldo + j;
+    if (ph.out64) static_cast<double *>(ph.out)[o] = X::dbl(v);
+    else X::st(ph.out, o, v);
+    if (sq) {
+      const double d = X::dbl(v);
+      *sq += d * d;
+    }
+  }
 }
 
 __device__ __forceinline__ int phase_tiles(const Phase &ph) {
@@ -383,8 +446,10 @@ __device__ __forceinline__ void run_phases(const Coop &cp, const Phase *ph, int 
   __shared__ __align__(16) unsigned char tsm[kTileBytes];
   __shared__ Phase sph[3];
   __syncthreads();  // the previous user of sph is done
-  if (threadIdx.x == 0)
-    for (int c = 0; c < count; ++c) sph[c] = ph[c];
+  static_assert(sizeof(Phase) % 8 == 0 && sizeof(Phase) / 8 <= NT, "a thread per word of a descriptor");
+  for (int c = 0; c < count; ++c)
+    if (threadIdx.x < sizeof(Phase) / 8)
+      reinterpret_cast<long long *>(&sph[c])[threadIdx.x] = reinterpret_cast<const long long *>(&ph[c])[threadIdx.x];
   __syncthreads();
   if constexpr (TCK) {  // large products on the tensor cores
     long long work = 0;
@@ -393,6 +458,14 @@ __device__ __forceinline__ void run_phases(const Coop &cp, const Phase *ph, int 
     if (cp.tc && work >= cp.tc->min_work) {
       run_phases_tc<R>(cp, sph, count, sq, reinterpret_cast<float2 *>(tsm));  // tsm: 32 KB staging
       return;
+    }
+  }
+  if (cp.size == 1) {  // small phases of a one-block chain directly
+    bool all = true;
+    for (int c = 0; c < count; ++c) all = all && use_direct(sph[c], 1);
+    if (all) {
+      for (int c = 0; c < count; ++c) phase_direct<R>(sph[c], sq);
+      return;  // (the caller's barrier follows)
     }
   }
   R *const base = reinterpret_cast<R *>(tsm);
@@ -436,18 +509,18 @@ __device__ __noinline__ void tc_tiles(const Coop &cp, const Phase &P, const Prod
                                       bool last, double *sq, float2 *stage) {
   const TcCtx &C = cp.tc->ctx;
   GemmSmem &S = *C.S;
-  const int m = P.m, n = P.n, K = P.k;
+  const int m = uniform(P.m), n = uniform(P.n), K = uniform(P.k);
   // scalars in registers: the MMA and copy loops read no memory between their
   // asm statements (which clobber memory)
-  const uint32_t tmem = C.tmem;
+  const uint32_t tmem = uniform(C.tmem);
   uint8_t *const dyn = C.dyn;
   const uint8_t *const asl = C.ws.asl, *const bsl = C.ws.bsl;
   const int *const rexp = C.ws.rexp, *const cexp = C.ws.cexp;
-  const int rank = cp.rank, size = cp.size;
+  const int rank = uniform(cp.rank), size = uniform(cp.size);
   const int ncb = (n + kGN - 1) / kGN, nks = (K + 15) / 16;
   const int ntiles = ((m + 127) / 128) * ncb;
   const int nch = (nks + kGChunk - 1) / kGChunk;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, w = uniform(tid >> 5), lane = tid & 31;
   // the barriers live for the whole kernel; the counts of the previous
   // products give each wait its phase
   const int fill0_copy = S.fill_copy, fill0_mma = S.fill_mma;
@@ -490,53 +563,55 @@ __device__ __noinline__ void tc_tiles(const Coop &cp, const Phase &P, const Prod
     }
   } else if (w == 1) {
     // ------------------------------------ MMA issue ------------------------------------
-    if (lane == 0) {
-      // instruction descriptors of N = 256, 192, 128, 64 (index 4 - N / 64)
-      const uint32_t id256 = idesc_bf16(256), id192 = idesc_bf16(192), id128 = idesc_bf16(128),
-                     id64 = idesc_bf16(64);
-      int fill = fill0_mma, ch = ch0_mma;
-      bool ok = true;
-      for (int t = rank; t < ntiles && ok; t += size) {
-        for (int ks = 0; ks < nks; ++ks, ++fill) {
-          const int kc = ks % kGChunk, b = ch & 1;
-          if (kc == 0 && ch >= 2) {  // the read-out of this buffer's previous chunk is done
-            if (!mbar_wait(&S.acc_empty[b], ((ch >> 1) - 1) & 1, stop)) {
-              tc_gave_up(cp, 2, ch);
-              ok = false;
-              break;
-            }
-          }
-          const int s = fill % kGStages, use = fill / kGStages;
-          if (!mbar_wait(&S.full[s], use & 1, stop)) {
-            tc_gave_up(cp, 3, fill);
+    // instruction descriptors of N = 256, 192, 128, 64
+    const uint32_t id256 = idesc_bf16(256), id192 = idesc_bf16(192), id128 = idesc_bf16(128),
+                   id64 = idesc_bf16(64);
+    const uint32_t dyn32 = uniform(su32(dyn));
+    int fill = uniform(fill0_mma), ch = uniform(ch0_mma);
+    bool ok = true;
+    for (int t = rank; t < ntiles && ok; t += size) {
+      for (int ks = 0; ks < nks; ++ks, ++fill) {
+        const int kc = ks % kGChunk, b = ch & 1;
+        if (kc == 0 && ch >= 2) {  // the read-out of this buffer's previous chunk is done
+          if (!mbar_wait_warp(&S.acc_empty[b], ((ch >> 1) - 1) & 1, stop)) {
+            if (lane == 0) tc_gave_up(cp, 2, ch);
             ok = false;
             break;
           }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = su32(dyn + s * kGStage), b0 = a0 + kGA;
-          const uint32_t d = tmem + b * kGSet;
-          const uint64_t B0 = smem_desc(b0);
-          // A_q against B_0 .. B_(3-q) (consecutive in shared memory) lands the
-          // orders q .. 3 at columns 64 q .. 192: one MMA per q; the first of a
-          // chunk starts the four sums afresh
-          mma_bf16(d, smem_desc(a0), B0, id256, kc == 0 ? 0u : 1u);
-          mma_bf16(d + 64, smem_desc(a0 + 4096), B0, id192, 1u);
-          mma_bf16(d + 128, smem_desc(a0 + 8192), B0, id128, 1u);
-          mma_bf16(d + 192, smem_desc(a0 + 12288), B0, id64, 1u);
-          // the order-4 products A_q B_(4-q) into the order-3 sum (FP32)
+        }
+        const int s = fill % kGStages, use = fill / kGStages;
+        if (!mbar_wait_warp(&S.full[s], use & 1, stop)) {
+          if (lane == 0) tc_gave_up(cp, 3, fill);
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = dyn32 + s * kGStage, b0 = a0 + kGA;
+        const uint32_t d = tmem + b * kGSet;
+        const uint64_t B0 = smem_desc(b0);
+        // A_q against B_0 .. B_(3-q) (consecutive in shared memory) lands the
+        // orders q .. 3 at columns 64 q .. 192: one MMA per q; the first of a
+        // chunk starts the four sums afresh
+        if (kc == 0) mma_bf16<false>(d, smem_desc(a0), B0, id256);
+        else mma_bf16<true>(d, smem_desc(a0), B0, id256);
+        mma_bf16<true>(d + 64, smem_desc(a0 + 4096), B0, id192);
+        mma_bf16<true>(d + 128, smem_desc(a0 + 8192), B0, id128);
+        mma_bf16<true>(d + 192, smem_desc(a0 + 12288), B0, id64);
+        // the order-4 products A_q B_(4-q) into the order-3 sum (FP32)
 #pragma unroll
-          for (int q = 0; q < kGS; ++q)
-            mma_bf16(d + 192, smem_desc(a0 + q * 4096), smem_desc(b0 + (4 - q) * 2048), id64, 1u);
-          mma_commit(&S.empty[s]);
-          if (kc == kGChunk - 1 || ks == nks - 1) {
-            mma_commit(&S.acc_full[b]);
-            ++ch;
-          }
+        for (int q = 0; q < kGS; ++q)
+          mma_bf16<true>(d + 192, smem_desc(a0 + q * 4096), smem_desc(b0 + (4 - q) * 2048), id64);
+        mma_commit(&S.empty[s]);
+        if (kc == kGChunk - 1 || ks == nks - 1) {
+          mma_commit(&S.acc_full[b]);
+          ++ch;
         }
       }
-      if (!ok) atomicExch((int *)stop, 1);
-      mma_commit(&S.fin);  // every MMA issued has completed when the call ends
-      mbar_wait(&S.fin, fins & 1);
+    }
+    if (!ok && lane == 0) atomicExch((int *)stop, 1);
+    mma_commit(&S.fin);  // every MMA issued has completed when the call ends
+    mbar_wait_warp(&S.fin, fins & 1);
+    if (lane == 0) {
       S.fill_mma = fill;
       S.chunk_mma = ch;
       S.fins = fins + 1;
@@ -814,11 +889,11 @@ __device__ void dense_forward(const DenseArgs &a, const Coop &cp) {
   BARRIER_OR_RETURN();
   {  // the range check |P|_F <= 4^kJmax (every block sums the partials in the same order)
     const double t = block_sum_of(a.red, cp.size);
-    double nrm = sqrt(t);
-    int j = 0;
-    while (nrm > 1.0 && j <= kJmax) { nrm *= 0.25; ++j; }
-    if (!(t == t) || isinf(t)) j = kJmax + 1;
-    if (threadIdx.x == 0) sh_jf = j;
+    if (threadIdx.x == 0) {  // (one warp: FP64 is scarce)
+      int j = 0;
+      for (double lim = 1.0; t > lim && j <= kJmax; lim *= 16.0) ++j;  // |P|_F^2 <= 16^j
+      sh_jf = (!(t == t) || isinf(t)) ? kJmax + 1 : j;
+    }
   }
   __syncthreads();
   const int JF = sh_jf;  // the doublings |P|_F alone would take
@@ -862,11 +937,15 @@ __device__ void dense_forward(const DenseArgs &a, const Coop &cp) {
     const double t1 = block_sum_of(a.red, cp.size);
     const double t2 = block_sum_of(a.red + cp.size, cp.size);
     const double t4 = block_sum_of(a.red + 2 * cp.size, cp.size);
-    double rho = fmin(sqrt(t1), fmin(sqrt(sqrt(t2)), sqrt(sqrt(sqrt(t4)))));
-    if (!(rho == rho)) rho = sqrt(t1);
-    int j = 0;
-    while (rho > 1.0 && j < JF) { rho *= 0.25; ++j; }
     if (threadIdx.x == 0) {
+      // the least j with |P|_F, |P^2|_F^(1/2) or |P^4|_F^(1/4) <= 4^j (squares
+      // compared; a NaN never satisfies its test)
+      int j = 0;
+      double l1 = 1.0, l2 = 1.0, l4 = 1.0;
+      while (j < JF && !(t1 <= l1) && !(t2 <= l2) && !(t4 <= l4)) {
+        l1 *= 16.0; l2 *= 256.0; l4 *= 65536.0;
+        ++j;
+      }
       sh_j = j;
       sh_sc = ldexp(1.0, -2 * j);
     }

@@ -61,7 +61,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *flags) {
 
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  // (a warp without contributions skips its FP64 additions, which are slow here)
+  if (__any_sync(0xffffffffu, (__double_as_longlong(v) << 1) != 0))
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   __syncthreads();
   if (l == 0) red[w] = v;
@@ -80,6 +82,7 @@ __device__ __forceinline__ double block_sum(double v) {
 
 // Sum of red[0, n) by the whole block; every thread gets the total.
 __device__ __forceinline__ double block_sum_of(const double *red, int n) {
+  if (n == 1) return red[0];
   double t = 0.0;
   for (int b = threadIdx.x; b < n; b += blockDim.x) t += red[b];
   return block_sum(t);

@@ -183,6 +183,7 @@ struct TcBatch {
   int *flags;          // status words: a bounded wait that gave up sets the timeout
   int grid;            // CTAs of the launch
   int max_nmc;         // largest number of orbital chunks of a job (density)
+  int two_acc;         // density: every system has at most 64 orbitals
 };
 
 // Float-pair potential pipeline of the mixed path (fftdf.cu): per system, the

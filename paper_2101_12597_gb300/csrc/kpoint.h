@@ -31,6 +31,16 @@ cudaError_t zgemm_sq(const double2 *A, int opa, const double2 *B, int opb, doubl
 // least (n = 129, 3 matrices: 52 us against 100; n = 64, 3: 32 against 12)
 inline bool oz_takes(int n, int batch) { return n >= 64 && (double)n * n * n * batch >= 3e6; }
 void oz_alloc(etdm_handle *h, int n, int batch);
+// one operand of a batched product by its vectors over K (rows of the first
+// factor, columns of the second): element (r, k) at p[r ld + k] when the
+// vectors are contiguous, else at p[k ld + r], conjugated if conj
+struct OzMat {
+  const double2 *p;
+  long stride;
+  int ld, rows_contiguous, conj;
+};
+cudaError_t oz_gemm(const OzWork &W, const OzMat &A, const OzMat &B, double2 *C, long sC, int ldc, int m,
+                    int n, int k, int batch, double alpha, double beta, int *flags, cudaStream_t s);
 cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const double2 *B, int opb,
                             double2 *C, int batch, double alpha, double beta, int *flags,
                             cudaStream_t s);

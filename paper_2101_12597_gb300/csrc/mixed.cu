@@ -370,7 +370,7 @@ constexpr int kRhoThreads = kRhoEpi + kRhoBld + 64;
 
 struct RhoBars {
   uint64_t tma_full[kRhoStages], bld_full[kRhoStages], empty[kRhoStages];
-  uint64_t acc_full, acc_empty, part_full, part_empty, fin;
+  uint64_t acc_full[2], acc_empty[2], part_full, part_empty, fin;
   uint32_t tbase;
   int stop;
   float2 part[kRhoParts - 1][kTP];
@@ -415,15 +415,17 @@ struct JobStream {
 __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
   extern __shared__ __align__(1024) uint8_t dsm[];
   __shared__ RhoBars R;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, w = uniform(tid >> 5), lane = tid & 31;
   if (tid == 0) {
     for (int s = 0; s < kRhoStages; ++s) {
       mbar_init(&R.tma_full[s], 1);
-      mbar_init(&R.bld_full[s], kRhoBld);
+      mbar_init(&R.bld_full[s], kRhoBldW);
       mbar_init(&R.empty[s], 1);
     }
-    mbar_init(&R.acc_full, 1);
-    mbar_init(&R.acc_empty, kRhoEpi);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&R.acc_full[b], 1);
+      mbar_init(&R.acc_empty[b], kRhoEpiW);
+    }
     mbar_init(&R.part_full, (kRhoParts - 1) * kTP);
     mbar_init(&R.part_empty, kTP);
     mbar_init(&R.fin, 1);
@@ -434,8 +436,12 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = R.tbase;
+  const uint32_t tmem = uniform(R.tbase);
   volatile int *stop = &R.stop;
+  // chunks of up to 64 orbitals leave tensor memory for two sets of the four
+  // accumulators, which alternate between jobs (the read-out of one overlaps
+  // the MMAs of the next)
+  const int nacc = B.two_acc ? 2 : 1;
 
   if (w == kRhoEpiW + kRhoBldW) {
     // ------------- bulk copies: X slices and the O-slice rows of each K step -------------
@@ -493,52 +499,55 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
     }
   } else if (w == kRhoEpiW + kRhoBldW + 1) {
     // ---------------------------------- MMA issue ----------------------------------
-    if (lane == 0) {
-      int fill = 0, jp = 0;  // jp: jobs run (the accumulator hand-overs)
-      bool ok = true;
-      JobStream js(B);
-      TcJob J;
-      while (ok && js.get(J)) {
-        if (!B.active[J.a.x]) continue;
-        const TcArgs &A = B.sys[J.a.x];
-        const int mc = J.a.z, nk = J.b.y;
-        const int nm = min(kNmax, A.Nocc - mc * kNmax);
-        const int nmpad = nm <= 32 ? 32 : ((nm + 31) / 32) * 32;
-        if (jp > 0 && !mbar_wait(&R.acc_empty, (jp - 1) & 1, stop)) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t idesc = idesc_bf16(nmpad), idesc2 = idesc_bf16(2 * nmpad);
-        for (int kk = 0; kk < nk; ++kk, ++fill) {
-          const int s = fill % kRhoStages, use = fill / kRhoStages;
-          if (!mbar_wait(&R.tma_full[s], use & 1, stop) || !mbar_wait(&R.bld_full[s], use & 1, stop)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = su32(dsm + s * kRhoStage), b0 = a0 + kRhoA;
-          uint64_t I[4], K[3];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) I[k] = smem_desc(a0 + k * kSlot);
-#pragma unroll
-          for (int k = 0; k < 3; ++k) K[k] = smem_desc(b0 + k * nmpad * 32);
-          // acc_o (order o) at column o * nmpad; I_i x [K_j; K_j+1] (N = 2 nmpad, the
-          // slices lie nmpad rows apart) adds I_i K_j to acc_(i+j) and I_i K_j+1 to
-          // acc_(i+j+1): the nine slice products of orders <= 3 in six MMAs
-          const uint32_t acc = kk > 0, ac = (uint32_t)nmpad;
-          mma_bf16(tmem, I[0], K[0], idesc2, acc);          // acc0 = I0 K0, acc1 = I0 K1
-          mma_bf16(tmem + 2 * ac, I[0], K[2], idesc, acc);  // acc2 = I0 K2
-          mma_bf16(tmem + ac, I[1], K[0], idesc2, 1u);      // acc1 += I1 K0, acc2 += I1 K1
-          mma_bf16(tmem + 3 * ac, I[1], K[2], idesc, acc);  // acc3 = I1 K2
-          mma_bf16(tmem + 2 * ac, I[2], K[0], idesc2, 1u);  // acc2 += I2 K0, acc3 += I2 K1
-          mma_bf16(tmem + 3 * ac, I[3], K[0], idesc, 1u);   // acc3 += I3 K0
-          mma_commit(&R.empty[s]);  // the stage is free once these MMAs complete
+    int fill = 0, jp = 0;  // jp: jobs run (the accumulator hand-overs)
+    bool ok = true;
+    JobStream js(B);
+    TcJob J;
+    while (ok && uniform((int)js.get(J))) {
+      if (!uniform(B.active[J.a.x])) continue;
+      const TcArgs &A = B.sys[J.a.x];
+      const int nm = uniform(min(kNmax, A.Nocc - J.a.z * kNmax)), nk = uniform(J.b.y);
+      const int nmpad = nm <= 32 ? 32 : ((nm + 31) / 32) * 32;
+      const int ab = jp & (nacc - 1), au = jp >> (nacc - 1);  // accumulator set, its uses before
+      if (au > 0 && !mbar_wait_warp(&R.acc_empty[ab], (au - 1) & 1, stop)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t idesc = idesc_bf16(nmpad), idesc2 = idesc_bf16(2 * nmpad);
+      // acc_o (order o) at column o * nmpad; I_i x [K_j; K_j+1] (N = 2 nmpad, the
+      // slices lie nmpad rows apart) adds I_i K_j to acc_(i+j) and I_i K_j+1 to
+      // acc_(i+j+1): the nine slice products of orders <= 3 in six MMAs
+      const uint32_t ac = (uint32_t)nmpad, acc0 = tmem + ab * (kTmemCols / 2);
+      const uint32_t acc1 = acc0 + ac, acc2 = acc1 + ac, acc3 = acc2 + ac;
+      for (int kk = 0; kk < nk; ++kk, ++fill) {
+        const int s = fill % kRhoStages, use = fill / kRhoStages;
+        if (!mbar_wait_warp(&R.tma_full[s], use & 1, stop) || !mbar_wait_warp(&R.bld_full[s], use & 1, stop)) {
+          ok = false;
+          break;
         }
-        if (ok) mma_commit(&R.acc_full);
-        ++jp;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = su32(dsm + s * kRhoStage), b0 = a0 + kRhoA;
+        const uint64_t I0 = smem_desc(a0), I1 = smem_desc(a0 + kSlot), I2 = smem_desc(a0 + 2 * kSlot),
+                       I3 = smem_desc(a0 + 3 * kSlot), K0 = smem_desc(b0), K2 = smem_desc(b0 + 2 * nmpad * 32);
+        if (kk == 0) {
+          mma_bf16<false>(acc0, I0, K0, idesc2);  // acc0 = I0 K0, acc1 = I0 K1
+          mma_bf16<false>(acc2, I0, K2, idesc);   // acc2 = I0 K2
+          mma_bf16<true>(acc1, I1, K0, idesc2);   // acc1 += I1 K0, acc2 += I1 K1
+          mma_bf16<false>(acc3, I1, K2, idesc);   // acc3 = I1 K2
+        } else {
+          mma_bf16<true>(acc0, I0, K0, idesc2);
+          mma_bf16<true>(acc2, I0, K2, idesc);
+          mma_bf16<true>(acc1, I1, K0, idesc2);
+          mma_bf16<true>(acc3, I1, K2, idesc);
+        }
+        mma_bf16<true>(acc2, I2, K0, idesc2);     // acc2 += I2 K0, acc3 += I2 K1
+        mma_bf16<true>(acc3, I3, K0, idesc);      // acc3 += I3 K0
+        mma_commit(&R.empty[s]);  // the stage is free once these MMAs complete
       }
-      if (!ok) atomicExch((int *)stop, 1);
-      mma_commit(&R.fin);  // every MMA issued has completed before the TMEM is released
-      mbar_wait(&R.fin, 0);
+      if (ok) mma_commit(&R.acc_full[ab]);
+      ++jp;
     }
+    if (!ok && lane == 0) atomicExch((int *)stop, 1);
+    mma_commit(&R.fin);  // every MMA issued has completed before the TMEM is released
+    mbar_wait_warp(&R.fin, 0);
   } else if (w >= kRhoEpiW) {
     // -------------- O-slice operand, B[m][a] = Oq[mu_a][m], from the gathered rows --------------
     const int bt = tid - kRhoEpi;
@@ -553,8 +562,18 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
       const int nm = min(kNmax, A.Nocc - mc * kNmax);
       const int ocw = A.ocw;  // staged row length (even)
       const int nmpad = nm <= 32 ? 32 : ((nm + 31) / 32) * 32;
+      // a thread per orbital: up to 64 orbitals take half of the threads, and
+      // two sets of them build consecutive K steps at the same time (a set
+      // arrives for both)
+      const int sets = nmpad <= kRhoBld / 2 ? 2 : 1;
+      const int bs = bt & (kRhoBld / sets - 1), set = bt / (kRhoBld / sets);
       for (int kk = 0; kk < nk; ++kk, ++fill) {
+        if ((fill & (sets - 1)) != set) continue;  // the other set's step
         const int s = fill % kRhoStages, use = fill / kRhoStages;
+        // the stage's previous use first (a set may have skipped it): a thread
+        // builds one of any three steps in a row, so the copies of the previous
+        // ring turn are issued and neither wait can take an older phase for its own
+        if (use > 0 && !mbar_wait(&R.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
         if (!mbar_wait(&R.tma_full[s], use & 1, stop)) { ok = false; break; }
         uint8_t *Bs = dsm + s * kRhoStage + kRhoA;
         const uint8_t *G = Bs + kRhoB;
@@ -563,7 +582,7 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
         // before the first use), laid out as the two 8-function halves of the
         // K step in each of the three slices
         const bool full = nrow == kKs;
-        for (int m = bt; m < nmpad; m += kRhoBld) {
+        for (int m = bs; m < nmpad; m += kRhoBld) {
           uint32_t w01[kKs], w2[kKs];
           if (full && m < nm) {
 #pragma unroll
@@ -598,7 +617,8 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(&R.bld_full[s]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive_n(&R.bld_full[s], sets);
       }
     }
     if (!ok) atomicExch((int *)stop, 1);
@@ -622,9 +642,11 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
       const int nmpad = nm <= 32 ? 32 : ((nm + 31) / 32) * 32;
       const int gp = tile_point(A.g, t, pe);
       const int ep = gp >= 0 ? (int)A.rowexp[gp] : 0;
-      ok = __all_sync(0xffffffffu, mbar_wait(&R.acc_full, jp & 1, stop));
+      const int ab = jp & (nacc - 1);
+      ok = __all_sync(0xffffffffu, mbar_wait(&R.acc_full[ab], (jp >> (nacc - 1)) & 1, stop));
       ++jp;
       if (!ok) break;
+      const uint32_t tacc = tmem + lanebits + ab * (kTmemCols / 2);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       // this warp's column part (a quarter of the chunk) in pieces of 8; the
       // column scales 2^g_m come from the (zero-padded) global array of the
@@ -633,12 +655,13 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
       const float *f = A.oscale + mc * kNmax;
       for (int c0 = cb; c0 < ce; c0 += 8) {
         uint32_t r[32];
-        tmem_ld_issue(tmem + lanebits + c0, r, nmpad);
+        tmem_ld_issue(tacc + c0, r, nmpad);
         tmem_ld_wait(r);
         rsum = rho_sum8(r, f + c0, rsum);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(&R.acc_empty);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&R.acc_empty[ab]);
       if (mc == J.a.w - 1) {  // the tile is done: add the column parts
         if (part > 0) {
           if (ntile > 0) ok = mbar_wait(&R.part_empty, (ntile - 1) & 1, stop);
@@ -679,9 +702,9 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
 // grid), those of orders 1 .. kVOrd into a second (about 2^-8 of the first, so
 // its FP32 rounding is 2^-32 of V's scale).  Two accumulator pairs (4 x 128 TMEM
 // columns) alternate between groups, so the read-out of one group overlaps the
-// MMAs of the next.  Warp roles: 0-15 read the accumulators (lane quarter
+// MMAs of the next.  Warp roles: 0-11 read the accumulators (lane quarter
 // w % 4, every fourth 8-column chunk by w / 4) and add into V by fixed-point
-// reductions; 16-23 build W from the X^T slices and v; 24 streams the X^T
+// reductions; 12-27 build W from the X^T slices and v; 28 streams the X^T
 // slices and the group buffers (v at the points, union entries); 25 issues the
 // MMAs.  Lane i takes the columns j <= i and adds into V[mu_j][mu_i]
 // (mu_j <= mu_i), so a warp's reductions run along a row of V.
@@ -689,7 +712,8 @@ constexpr int kVA = kVSlW * kSlot;  // W slices (128 rows)
 constexpr int kVB = kVSlX * kSlot;  // X^T slices (np rows each, packed as stored)
 constexpr int kVStage = kVA + kVB;
 constexpr int kVStages = (200 * 1024) / kVStage;  // operand ring in 200 KB of shared memory
-constexpr int kVEpiW = 16, kVBldW = 8;  // warps: 0-15 read-out, 16-23 build W
+constexpr int kVEpiW = 12, kVBldW = 16;  // warps: 0-11 read-out, 12-27 build W
+constexpr int kVParts = kVEpiW / 4;      // column parts of the read-out per lane quarter
 constexpr int kVEpi = kVEpiW * 32, kVBld = kVBldW * 32;
 constexpr int kVThreads = kVEpi + kVBld + 64;
 // tiles per V group at most (the group size is chosen per handle, <= this):
@@ -735,11 +759,11 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
   extern __shared__ __align__(1024) uint8_t dsm[];
   uint8_t *tbuf = dsm + kVStages * kVStage;  // 2 group buffers: vt[nt * 128] float2, vent[np] float4
   __shared__ VBars R;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, w = uniform(tid >> 5), lane = tid & 31;
   if (tid == 0) {
     for (int s = 0; s < kVStages; ++s) {
       mbar_init(&R.tma_full[s], 1);
-      mbar_init(&R.bld_full[s], kVBld);
+      mbar_init(&R.bld_full[s], kVBldW);
       mbar_init(&R.empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -756,7 +780,7 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = R.tbase;
+  const uint32_t tmem = uniform(R.tbase);
   // each CTA's jobs are a contiguous run of groups (of one system or a few):
   // CTAs running at the same time work in different parts of a box and rarely
   // add into the same entries of V
@@ -798,53 +822,59 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
     }
   } else if (w == kVEpiW + kVBldW + 1) {
     // ---------------------------------- MMA issue ----------------------------------
-    if (lane == 0) {
-      int fill = 0, it = 0;
-      bool ok = true;
-      JobStream js(B);
-      TcJob J;
-      for (; ok && js.get(J); ++it) {
-        if (!B.active[J.a.x]) { --it; continue; }
-        const int buf = it & 1;
-        const int nt = J.a.w, np = J.b.y;
-        // the accumulator pair of group it - 2 has been read
-        if (it >= 2 && !mbar_wait(&R.acc_empty[buf], ((it >> 1) - 1) & 1, stop)) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t idesc = idesc_bf16(np);
-        const uint32_t d0 = tmem + buf * 2 * kNmax, d1 = d0 + kNmax;
-        for (int kk = 0; kk < nt * kSteps; ++kk, ++fill) {
-          const int s = fill % kVStages, use = fill / kVStages;
-          if (!mbar_wait(&R.tma_full[s], use & 1, stop) || !mbar_wait(&R.bld_full[s], use & 1, stop)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = su32(dsm + s * kVStage), b0 = a0 + kVA;
-          uint64_t W[kVSlW], X[kVSlX];
-#pragma unroll
-          for (int k = 0; k < kVSlW; ++k) W[k] = smem_desc(a0 + k * kSlot);
-#pragma unroll
-          for (int k = 0; k < kVSlX; ++k) X[k] = smem_desc(b0 + k * np * 32);
-          const uint32_t acc = kk > 0;
-          mma_bf16(d0, W[0], X[0], idesc, acc);  // order 0
-#pragma unroll
-          for (int o = 1; o <= kVOrd; ++o)        // orders 1 .. kVOrd (W0 X1 first)
-#pragma unroll
-            for (int q = 0; q <= o; ++q)
-              if (q < kVSlW && o - q < kVSlX)
-                mma_bf16(d1, W[q], X[o - q], idesc, (o == 1 && q == 0) ? acc : 1u);
-          mma_commit(&R.empty[s]);
+    int fill = 0, it = 0;
+    bool ok = true;
+    JobStream js(B);
+    TcJob J;
+    for (; ok && uniform((int)js.get(J)); ++it) {
+      if (!uniform(B.active[J.a.x])) { --it; continue; }
+      const int buf = it & 1;
+      const int nt = uniform(J.a.w), np = uniform(J.b.y);
+      // the accumulator pair of group it - 2 has been read
+      if (it >= 2 && !mbar_wait_warp(&R.acc_empty[buf], ((it >> 1) - 1) & 1, stop)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t idesc = idesc_bf16(np);
+      const uint32_t d0 = tmem + buf * 2 * kNmax, d1 = d0 + kNmax;
+      for (int kk = 0; kk < nt * kSteps; ++kk, ++fill) {
+        const int s = fill % kVStages, use = fill / kVStages;
+        if (!mbar_wait_warp(&R.tma_full[s], use & 1, stop) || !mbar_wait_warp(&R.bld_full[s], use & 1, stop)) {
+          ok = false;
+          break;
         }
-        if (ok) mma_commit(&R.acc_full[buf]);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = su32(dsm + s * kVStage), b0 = a0 + kVA;
+        uint64_t W[kVSlW], X[kVSlX];
+#pragma unroll
+        for (int k = 0; k < kVSlW; ++k) W[k] = smem_desc(a0 + k * kSlot);
+#pragma unroll
+        for (int k = 0; k < kVSlX; ++k) X[k] = smem_desc(b0 + k * np * 32);
+        if (kk == 0) {
+          mma_bf16<false>(d0, W[0], X[0], idesc);  // order 0
+          mma_bf16<false>(d1, W[0], X[1], idesc);  // orders 1 .. kVOrd (W0 X1 first)
+        } else {
+          mma_bf16<true>(d0, W[0], X[0], idesc);
+          mma_bf16<true>(d1, W[0], X[1], idesc);
+        }
+#pragma unroll
+        for (int o = 1; o <= kVOrd; ++o)
+#pragma unroll
+          for (int q = 0; q <= o; ++q)
+            if (q < kVSlW && o - q < kVSlX && !(o == 1 && q == 0)) mma_bf16<true>(d1, W[q], X[o - q], idesc);
+        mma_commit(&R.empty[s]);
       }
-      if (!ok) atomicExch((int *)stop, 1);
-      mma_commit(&R.fin);
-      mbar_wait(&R.fin, 0);
+      if (ok) mma_commit(&R.acc_full[buf]);
     }
+    if (!ok && lane == 0) atomicExch((int *)stop, 1);
+    mma_commit(&R.fin);
+    mbar_wait_warp(&R.fin, 0);
   } else if (w >= kVEpiW) {
     // -------------------- W = (v X)^T: rows b, 8 points of each K step ----------------------
+    // A K step takes 2 x 128, 2 x 64 or 2 x 32 threads (rows of the union, 8
+    // points each), so 2, 4 or 8 sets of them build consecutive K steps at the
+    // same time: a step's chain of wait, loads, slices and fence is what bounds
+    // the pass (about 1200 cycles a step with one set, whatever the union's
+    // size).  A set arrives for all of them.
     const int bt = tid - kVEpi;
-    const int b = bt & 127, h = bt >> 7;
     int fill = 0, it = 0;
     bool ok = true;
     JobStream js(B);
@@ -853,6 +883,9 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
       if (!B.active[J.a.x]) { --it; continue; }
       const int mb = it & 1;
       const int nt = J.a.w, np = J.b.y, nu = J.b.z;
+      const int rl = nu > 64 ? 7 : nu > 32 ? 6 : 5;  // log2 rows of a set
+      const int b = bt & ((1 << rl) - 1), h = (bt >> rl) & 1;
+      const int sets = kVBld >> (rl + 1), set = bt >> (rl + 1);
       ok = __all_sync(0xffffffffu, mbar_wait(&R.tile_full[mb], (it >> 1) & 1, stop));
       if (!ok) break;
       const uint8_t *tb = tbuf + mb * kVTileBuf;
@@ -867,14 +900,19 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
         sb = pow2f(8 - slice_exp(e.z * vmax * 1.0001f)) * e.y;
       }
       for (int kk = 0; kk < nt * kSteps; ++kk, ++fill) {
+        if ((fill & (sets - 1)) != set) continue;  // another set's step
         const int s = fill % kVStages, use = fill / kVStages;
+        // the stage's previous use first: a set may have skipped uses of the
+        // stage (the sets change between jobs).  The copies of every step
+        // before this one's ring turn are issued by now (the job's buffers or
+        // the set's last step say so), so the use before the previous one is
+        // complete and neither wait can take an older phase for its own.
         if (use > 0 && !mbar_wait(&R.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
         if (!mbar_wait(&R.tma_full[s], use & 1, stop)) { ok = false; break; }
         uint8_t *Ast = dsm + s * kVStage;
         const uint8_t *Bst = Ast + kVA;
         const int off = kstep_off(b, h * 8);
-        uint4 o[kVSlW];
-        if (b < nu) {
+        if (b < nu) {  // (rows beyond the union feed accumulator lanes nobody reads)
           uint4 xs[kVSlX];
 #pragma unroll
           for (int k = 0; k < kVSlX; ++k) xs[k] = *(const uint4 *)(Bst + k * np * 32 + off);
@@ -899,15 +937,12 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
             for (int k = 0; k < kVSlW; ++k) ww[k][u] = pack_bf16(r[0][k], r[1][k]);
           }
 #pragma unroll
-          for (int k = 0; k < kVSlW; ++k) o[k] = make_uint4(ww[k][0], ww[k][1], ww[k][2], ww[k][3]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < kVSlW; ++k) o[k] = make_uint4(0u, 0u, 0u, 0u);
+          for (int k = 0; k < kVSlW; ++k)
+            *(uint4 *)(Ast + k * kSlot + off) = make_uint4(ww[k][0], ww[k][1], ww[k][2], ww[k][3]);
         }
-#pragma unroll
-        for (int k = 0; k < kVSlW; ++k) *(uint4 *)(Ast + k * kSlot + off) = o[k];
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(&R.bld_full[s]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive_n(&R.bld_full[s], sets);
       }
       ok = __all_sync(0xffffffffu, ok);
       if (lane == 0) mbar_arrive(&R.tile_empty[mb]);
@@ -915,7 +950,7 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
     if (!ok) atomicExch((int *)stop, 1);
   } else {
     // ------------------------- accumulator read-out into V ----------------------------
-    // lane i of quarter w % 4 holds row i; columns j <= i of every fourth
+    // lane i of quarter w % 4 holds row i; columns j <= i of every kVParts-th
     // 8-column chunk (by w / 4): y = acc0 + acc1 as a float pair, scaled to the
     // fixed-point unit, added into V[mu_j][mu_i]
     const int quad = w & 3, part = w >> 2;
@@ -946,7 +981,7 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
       unsigned long long *const vrow = A.Vfix + mui;
       const uint32_t t0 = tmem + lanebits + buf * 2 * kNmax;
       const int jend = quad * 32 < nu ? min(quad * 32 + 32, nu) : 0;
-      for (int c0 = part * 8; c0 < jend; c0 += 32) {
+      for (int c0 = part * 8; c0 < jend; c0 += 8 * kVParts) {
         uint32_t ra[16];
         tmem_ld2_issue(t0 + c0, t0 + kNmax + c0, ra);
         tmem_ld2_wait(ra);
@@ -1013,25 +1048,36 @@ __global__ void tables_f32_kernel(const double *sq, const double *ex, const doub
 // chain): g_m = ilogb(max_mu |O_mu,m|) + 2, K0 + K1 + K2 = O 2^(8 - g) to 24 bits
 // (K_k on the 2^-8k grid); dO = O - Oq (FP64) for the first-order energy
 // correction sum (4 H O) o dO.
-// O slicing, the first of two coalesced passes over the row-major O: the
-// largest |O| of each column (orbital), as the bits of a non-negative double
-// (which order as integers); a warp takes 32 consecutive columns over a run
-// of 64 rows.  omax is zero on entry.
+// O slicing, the first of two coalesced passes over the row-major O: a float
+// with the exponent of the largest |O| of each column (orbital), as its bits
+// (which order as integers).  The exponent is all the slices need: |hi|, one
+// step down when lo has the other sign, has that of |hi + lo| (FP64 sums and
+// maxima took 37 us at M = 256, N = 128 for 0.3 MB).  A warp takes 32
+// consecutive columns over a run of kOmaxRows rows.  omax is zero on entry.
+constexpr int kOmaxRows = 16;
 __global__ void __launch_bounds__(256) omax_kernel(const OsArgs *av, const int *active) {
   if (!active[blockIdx.y]) return;
   const OsArgs &a = av[blockIdx.y];
   const int M = a.M, N = a.N;
-  const int ncg = (N + 31) / 32, nrc = (M + 63) / 64;
+  const int ncg = (N + 31) / 32, nrc = (M + kOmaxRows - 1) / kOmaxRows;
   const long items = (long)ncg * nrc;
   const int lane = threadIdx.x & 31;
   const long wstride = ((long)gridDim.x * blockDim.x) >> 5;
   for (long w = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < items; w += wstride) {
-    const int m = (int)(w % ncg) * 32 + lane, r0 = (int)(w / ncg) * 64;
+    const int m = (int)(w % ncg) * 32 + lane, r0 = (int)(w / ncg) * kOmaxRows;
     if (m >= N) continue;
-    const int r1 = min(r0 + 64, M);
-    double mx = 0.0;
-    for (int r = r0; r < r1; ++r) mx = fmax(mx, fabs(pair::to_double(a.O[(long)r * N + m])));
-    atomicMax(a.omax + m, (unsigned long long)__double_as_longlong(mx));
+    float2 o[kOmaxRows];
+#pragma unroll
+    for (int r = 0; r < kOmaxRows; ++r)
+      o[r] = r0 + r < M ? a.O[(long)(r0 + r) * N + m] : make_float2(0.f, 0.f);
+    unsigned mx = 0u;
+#pragma unroll
+    for (int r = 0; r < kOmaxRows; ++r) {
+      const unsigned f = __float_as_uint(fabsf(o[r].x));
+      const bool less = o[r].y != 0.f && ((__float_as_uint(o[r].x) ^ __float_as_uint(o[r].y)) >> 31);
+      mx = max(mx, f - (less && f > 0u ? 1u : 0u));
+    }
+    atomicMax(a.omax + m, (unsigned long long)mx);
   }
 }
 
@@ -1045,8 +1091,8 @@ __global__ void __launch_bounds__(256) oslice_kernel(const OsArgs *av, const int
   const long MN = (long)M * N;
   for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < MN; e += (long)gridDim.x * blockDim.x) {
     const int r = (int)(e / N), m = (int)(e % N);
-    const double mx = __longlong_as_double((long long)a.omax[m]);
-    const int g = mx > 0.0 ? ilogb(mx) + 2 : 0;
+    const float mx = __uint_as_float((unsigned)a.omax[m]);
+    const int g = mx > 0.f ? ilogbf(mx) + 2 : 0;
     if (r == 0) a.oscale[m] = ldexpf(1.f, g);
     const double o = pair::to_double(a.O[e]);
     const double t0 = ldexp(o, 8 - g);
@@ -1165,7 +1211,7 @@ cudaError_t launch_mixed_rho(const MixedPlan &P, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(P.omax, 0, P.omax_bytes, s);
   if (e != cudaSuccess) return e;
   {
-    const long warps = (long)((P.os_maxN + 31) / 32) * ((P.os_maxMN / std::max(P.os_maxN, 1) + 63) / 64);
+    const long warps = (long)((P.os_maxN + 31) / 32) * ((P.os_maxMN / std::max(P.os_maxN, 1) + kOmaxRows - 1) / kOmaxRows);
     const int bx = (int)std::max<long>(1, std::min<long>((warps + 7) / 8, 4096));
     omax_kernel<<<dim3(bx, P.n_sys), 256, 0, s>>>(P.os, P.active);
     const int bs = (int)std::max<long>(1, std::min<long>((P.os_maxMN + 255) / 256, 4096));

@@ -42,22 +42,18 @@
 #include "device.cuh"
 #include "host.h"
 #include "kpoint.h"
+#include "ozdigits.cuh"
 #include "tc.cuh"
 
 namespace etdm {
 
-constexpr int kOzS = 8;                        // base-256 digits per operand
 constexpr int kOzRows = 128, kOzCols = 64;     // real output tile
 constexpr int kOzA = kOzS * kOzRows * 32;      // A digits of a K step of 16 (32 KB)
 constexpr int kOzB = kOzS * kOzCols * 32;      // B digits of a K step (16 KB)
 constexpr int kOzStage = kOzA + kOzB;
 constexpr int kOzStages = 4;
-constexpr int kOzChunk = 10;                   // K steps between read-outs
 constexpr int kOzEpiW = 16;                    // read-out warps (lane quarter w % 4, columns 16 (w / 4))
 constexpr int kOzThreads = (kOzEpiW + 2) * 32;
-constexpr int kOzBad = 0x7ff;                  // exponent field of a row with an infinity or NaN
-
-static_assert(6LL * kOzChunk * 16 * 128 * 128 <= (1LL << 24), "orders 0-5 of a chunk are exact in FP32");
 
 struct OzArgs {
   const uint8_t *asl, *bsl;   // [batch][row block][K step][digit][4 KB], [batch][column block]...[2 KB]
@@ -68,34 +64,6 @@ struct OzArgs {
   double alpha, beta;
   int *flags;
 };
-
-// ---- digits -------------------------------------------------------------------
-__device__ __forceinline__ int exp_field(double x) { return (int)((__double2hiint(x) >> 20) & 0x7ff); }
-
-// round(x 2^(1084 - bmax)) for |x| < 2^(bmax - 1022), plus 128 in every byte:
-// byte 7 - t is digit t + 128
-__device__ __forceinline__ unsigned long long biased_digits(double x, int bmax) {
-  const long long b = __double_as_longlong(x);
-  const int f = (int)((b >> 52) & 0x7ff);
-  long long m = b & 0xfffffffffffffLL;
-  m |= f ? (1LL << 52) : 0;
-  const int sh = 9 - (bmax - max(f, 1));
-  if (sh >= 0) {
-    m <<= sh;
-  } else {
-    const int r = min(-sh, 63);
-    m = (m + (1LL << (r - 1))) >> r;
-  }
-  if (b < 0) m = -m;
-  return (unsigned long long)m + 0x8080808080808080ULL;
-}
-
-// digit t as a float (exact)
-template <int T>
-__device__ __forceinline__ float digit(unsigned long long y) {
-  const uint32_t w = T < 4 ? (uint32_t)(y >> 32) : (uint32_t)y;
-  return __fsub_rn(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440 + (3 - (T & 3)))), 8388736.f);
-}
 
 // Digits of one operand.  ROWC: the elements of a row are contiguous in memory
 // (a block takes 8 rows, a warp per row for the maxima), else the rows are
@@ -173,8 +141,8 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const double2 *Xb, long s
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      yr[q] = biased_digits(z[q].x, bm);
-      yi[q] = biased_digits(conj ? -z[q].y : z[q].y, bm);
+      yr[q] = biased(to_fixed(z[q].x, bm));
+      yi[q] = biased(to_fixed(conj ? -z[q].y : z[q].y, bm));
     }
     uint8_t *blk = base + (long)(g >> 1) * (kOzS * (ISB ? kOzCols : kOzRows) * 32);
     const int h = (g & 1) * 8;
@@ -197,28 +165,10 @@ struct OzBars {
   int stop;
 };
 
-// 4 columns of the eight accumulators (64 columns apart) of a lane quarter
-__device__ __forceinline__ void oz_ld_issue(uint32_t t, uint32_t (&r)[32]) {
-#pragma unroll
-  for (int o = 0; o < 8; ++o)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[4 * o]), "=r"(r[4 * o + 1]), "=r"(r[4 * o + 2]), "=r"(r[4 * o + 3])
-                 : "r"(t + o * kOzCols));
-}
-
-__device__ __forceinline__ int oz_int(uint32_t bits) { return __float2int_rn(__uint_as_float(bits)); }
-
-// v 2^e without intermediate overflow or double rounding in the normal range
-__device__ __forceinline__ double oz_scale(double v, int e) {
-  const int f = exp_field(v) + e;
-  if (f > 0 && f < 0x7ff && exp_field(v) > 0) return __hiloint2double(__double2hiint(v) + e * (1 << 20), __double2loint(v));
-  return v == 0.0 ? 0.0 : scalbn(v, e);
-}
-
 __global__ void __launch_bounds__(kOzThreads, 1) oz_product_kernel(OzArgs g) {
   extern __shared__ __align__(1024) uint8_t dsm[];
   __shared__ OzBars S;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, w = uniform(tid >> 5), lane = tid & 31;
   if (tid == 0) {
     for (int s = 0; s < kOzStages; ++s) {
       mbar_init(&S.full[s], 1);
@@ -234,7 +184,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_product_kernel(OzArgs g) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = S.tbase;
+  const uint32_t tmem = uniform(S.tbase);
   volatile int *stop = &S.stop;
   const int per = g.nrb * g.ncb, ntiles = per * g.batch, nks = g.nks;
 
@@ -263,42 +213,46 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_product_kernel(OzArgs g) {
     }
   } else if (w == kOzEpiW + 1) {
     // --------------------------------- MMA issue ---------------------------------
-    if (lane == 0) {
-      const uint32_t id256 = idesc_bf16(256), id192 = idesc_bf16(192), id128 = idesc_bf16(128),
-                     id64 = idesc_bf16(64);
-      int fill = 0, ch = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        for (int ks = 0; ks < nks; ++ks, ++fill) {
-          const bool fresh = ks % kOzChunk == 0;
-          if (fresh && ch > 0 && !mbar_wait(&S.acc_empty, (ch - 1) & 1, stop)) { ok = false; break; }
-          const int s = fill % kOzStages, use = fill / kOzStages;
-          if (!mbar_wait(&S.full[s], use & 1, stop)) { ok = false; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = su32(dsm + s * kOzStage), b0 = a0 + kOzA;
-          // digit q of A times digits 0 .. 7 - q of B (consecutive rows in
-          // shared memory) adds into the orders q .. 7 (consecutive columns)
-          const uint64_t B0 = smem_desc(b0), B4 = smem_desc(b0 + 4 * kOzCols * 32);
+    const uint32_t id256 = idesc_bf16(256), id192 = idesc_bf16(192), id128 = idesc_bf16(128),
+                   id64 = idesc_bf16(64);
+    int fill = 0, ch = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      for (int ks = 0; ks < nks; ++ks, ++fill) {
+        const bool fresh = ks % kOzChunk == 0;
+        if (fresh && ch > 0 && !mbar_wait_warp(&S.acc_empty, (ch - 1) & 1, stop)) { ok = false; break; }
+        const int s = fill % kOzStages, use = fill / kOzStages;
+        if (!mbar_wait_warp(&S.full[s], use & 1, stop)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = su32(dsm + s * kOzStage), b0 = a0 + kOzA;
+        // digit q of A times digits 0 .. 7 - q of B (consecutive rows in
+        // shared memory) adds into the orders q .. 7 (consecutive columns)
+        const uint64_t B0 = smem_desc(b0), B4 = smem_desc(b0 + 4 * kOzCols * 32);
+        if (fresh) {
+          mma_bf16<false>(tmem, smem_desc(a0), B0, id256);
+          mma_bf16<false>(tmem + 256, smem_desc(a0), B4, id256);
+        } else {
+          mma_bf16<true>(tmem, smem_desc(a0), B0, id256);
+          mma_bf16<true>(tmem + 256, smem_desc(a0), B4, id256);
+        }
 #pragma unroll
-          for (int q = 0; q < kOzS; ++q) {
-            const uint64_t A = smem_desc(a0 + q * kOzRows * 32);
-            const uint32_t d = tmem + q * kOzCols, acc = (fresh && q == 0) ? 0u : 1u;
-            const int nc = kOzS - q;  // digits of B
-            mma_bf16(d, A, B0, nc >= 4 ? id256 : nc == 3 ? id192 : nc == 2 ? id128 : id64, acc);
-            if (nc > 4)
-              mma_bf16(d + 256, A, B4, nc == 8 ? id256 : nc == 7 ? id192 : nc == 6 ? id128 : id64, acc);
-          }
-          mma_commit(&S.empty[s]);
-          if (ks % kOzChunk == kOzChunk - 1 || ks == nks - 1) {
-            mma_commit(&S.acc_full);
-            ++ch;
-          }
+        for (int q = 1; q < kOzS; ++q) {
+          const uint64_t A = smem_desc(a0 + q * kOzRows * 32);
+          const uint32_t d = tmem + q * kOzCols;
+          const int nc = kOzS - q;  // digits of B
+          mma_bf16<true>(d, A, B0, nc >= 4 ? id256 : nc == 3 ? id192 : nc == 2 ? id128 : id64);
+          if (nc > 4) mma_bf16<true>(d + 256, A, B4, nc == 7 ? id192 : nc == 6 ? id128 : id64);
+        }
+        mma_commit(&S.empty[s]);
+        if (ks % kOzChunk == kOzChunk - 1 || ks == nks - 1) {
+          mma_commit(&S.acc_full);
+          ++ch;
         }
       }
-      if (!ok) atomicExch((int *)stop, 1);
-      mma_commit(&S.fin);  // every MMA issued has completed before the TMEM is released
-      mbar_wait(&S.fin, 0);
     }
+    if (!ok && lane == 0) atomicExch((int *)stop, 1);
+    mma_commit(&S.fin);  // every MMA issued has completed before the TMEM is released
+    mbar_wait_warp(&S.fin, 0);
   } else {
     // ------------------------- read-out and outputs -------------------------
     const int quad = w & 3, part = w >> 2;
@@ -318,7 +272,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_product_kernel(OzArgs g) {
 #pragma unroll
         for (int cg = 0; cg < 4; ++cg) {
           uint32_t r[32];
-          oz_ld_issue(tbase + cg * 4, r);
+          oz_ld_issue(tbase + cg * 4, r, kOzCols);
           tmem_ld_wait(r);
           if (cg == 3) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -326,14 +280,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_product_kernel(OzArgs g) {
             if (lane == 0) mbar_arrive(&S.acc_empty);
           }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            // orders 0-3: |i0 256 + i1|, |i2 256 + i3| < 2^31 (see the chunk bound)
-            const int j01 = oz_int(r[j]) * 256 + oz_int(r[4 + j]);
-            const int j23 = oz_int(r[8 + j]) * 256 + oz_int(r[12 + j]);
-            hi[cg * 4 + j] += (long long)j01 * 65536 + j23;
-            lo[cg * 4 + j] += (long long)oz_int(r[16 + j]) * 16777216 + (long long)oz_int(r[20 + j]) * 65536 +
-                              (long long)oz_int(r[24 + j]) * 256 + oz_int(r[28 + j]);
-          }
+          for (int j = 0; j < 4; ++j) oz_add(r, j, hi[cg * 4 + j], lo[cg * 4 + j]);
         }
       }
       if (!ok) break;
@@ -380,16 +327,17 @@ size_t oz_b_bytes(int n) { return (size_t)((2 * n + kOzCols - 1) / kOzCols) * oz
 int oz_rows_pad(int n, int q) { return (n + q - 1) / q * q; }
 
 template <bool ISB>
-cudaError_t oz_slice(const double2 *X, int n, int contiguous, int conj, int batch, uint8_t *dst,
-                     int *exps, cudaStream_t s) {
+cudaError_t oz_slice(const OzMat &X, int b0, int rows, int k, int batch, uint8_t *dst, int *exps,
+                     cudaStream_t s) {
   constexpr int BR = ISB ? kOzCols / 2 : kOzRows;
-  const int nblk = (n + BR - 1) / BR, nks = oz_ksteps(n);
-  if (contiguous)
-    oz_slice_kernel<true, ISB><<<dim3(nblk * BR / 8, batch), 256, 0, s>>>(
-        X, (long)n * n, n, n, n, conj, dst, exps, nblk, nks);
+  const int nblk = (rows + BR - 1) / BR, nks = oz_ksteps(k);
+  const double2 *p = X.p + b0 * X.stride;
+  if (X.rows_contiguous)
+    oz_slice_kernel<true, ISB><<<dim3(nblk * BR / 8, batch), 256, 0, s>>>(p, X.stride, X.ld, rows, k, X.conj,
+                                                                          dst, exps, nblk, nks);
   else
-    oz_slice_kernel<false, ISB><<<dim3(nblk * BR / 16, batch), 256, 0, s>>>(
-        X, (long)n * n, n, n, n, conj, dst, exps, nblk, nks);
+    oz_slice_kernel<false, ISB><<<dim3(nblk * BR / 16, batch), 256, 0, s>>>(p, X.stride, X.ld, rows, k, X.conj,
+                                                                            dst, exps, nblk, nks);
   return cudaGetLastError();
 }
 }  // namespace
@@ -416,26 +364,23 @@ void oz_alloc(etdm_handle *h, int n, int batch) {
   W.cexp = W.rexp + (size_t)W.group * oz_rows_pad(n, kOzRows);
 }
 
-// C = alpha op(A) op(B) + beta C for a batch of n x n matrices (n = W.n)
-cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const double2 *B, int opb,
-                            double2 *C, int batch, double alpha, double beta, int *flags,
-                            cudaStream_t s) {
-  const int n = W.n;
-  const long nn = (long)n * n;
+// C = alpha A B + beta C over a batch, A m x k by rows, B n x k by the columns of
+// the product's second factor (m, n, k <= W.n)
+cudaError_t oz_gemm(const OzWork &W, const OzMat &A, const OzMat &B, double2 *C, long sC, int ldc, int m,
+                    int n, int k, int batch, double alpha, double beta, int *flags, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(oz_product_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kOzStages * kOzStage);
   if (e != cudaSuccess) return e;
   for (int b0 = 0; b0 < batch; b0 += W.group) {
     const int nb = std::min(W.group, batch - b0);
-    // op(A) rows: contiguous for A, columns of A for A^dagger; op(B) columns
-    if ((e = oz_slice<false>(A + b0 * nn, n, opa == 0, opa, nb, W.a, W.rexp, s)) != cudaSuccess) return e;
-    if ((e = oz_slice<true>(B + b0 * nn, n, opb != 0, opb, nb, W.b, W.cexp, s)) != cudaSuccess) return e;
+    if ((e = oz_slice<false>(A, b0, m, k, nb, W.a, W.rexp, s)) != cudaSuccess) return e;
+    if ((e = oz_slice<true>(B, b0, n, k, nb, W.b, W.cexp, s)) != cudaSuccess) return e;
     OzArgs g{};
     g.asl = W.a; g.bsl = W.b; g.rexp = W.rexp; g.cexp = W.cexp;
-    g.C = C + b0 * nn; g.sC = nn;
-    g.m = n; g.n = n; g.ldc = n;
-    g.nks = oz_ksteps(n);
-    g.nrb = (n + kOzRows - 1) / kOzRows;
+    g.C = C + b0 * sC; g.sC = sC;
+    g.m = m; g.n = n; g.ldc = ldc;
+    g.nks = oz_ksteps(k);
+    g.nrb = (m + kOzRows - 1) / kOzRows;
     g.ncb = (2 * n + kOzCols - 1) / kOzCols;
     g.batch = nb;
     g.alpha = alpha; g.beta = beta;
@@ -445,6 +390,17 @@ cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const do
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+// C = alpha op(A) op(B) + beta C for a batch of n x n matrices (n = W.n)
+cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const double2 *B, int opb,
+                            double2 *C, int batch, double alpha, double beta, int *flags,
+                            cudaStream_t s) {
+  const int n = W.n;
+  const long nn = (long)n * n;
+  // rows of op(A): contiguous for A, columns of A for A^dagger; columns of op(B)
+  return oz_gemm(W, OzMat{A, nn, n, opa == 0, opa}, OzMat{B, nn, n, opb != 0, opb}, C, nn, n, n, n, n, batch,
+                 alpha, beta, flags, s);
 }
 
 }  // namespace etdm

@@ -106,7 +106,8 @@ void build_mixed_plan(etdm_handle *owner, const std::vector<etdm_handle *> &subs
       ptr[b + 1] = (int)jobs.size();
     }
     P->rho = TcBatch{d_tc, dupload(owner, jobs.data(), jobs.size()),
-                     dupload(owner, ptr.data(), ptr.size()), d_active, d_flags, grid, max_nmc};
+                     dupload(owner, ptr.data(), ptr.size()), d_active, d_flags, grid, max_nmc,
+                     P->os_maxN <= 64};
   }
 
   // V: per CTA a contiguous run of (system, group)
@@ -141,7 +142,7 @@ void build_mixed_plan(etdm_handle *owner, const std::vector<etdm_handle *> &subs
       ptr[grid] = (int)nj;
     }
     P->v = TcBatch{d_tc, dupload(owner, jobs.data(), jobs.size()),
-                   dupload(owner, ptr.data(), ptr.size()), d_active, d_flags, grid, 1};
+                   dupload(owner, ptr.data(), ptr.size()), d_active, d_flags, grid, 1, 0};
   }
   P->vf_blocks = (int)std::min<long>(1024, (maxMM + 255) / 256);
   P->vfix = vfix;

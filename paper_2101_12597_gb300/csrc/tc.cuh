@@ -37,27 +37,44 @@ __device__ __forceinline__ uint32_t idesc_bf16(int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                         uint32_t accumulate) {
+// The issuing warp runs its loop as a whole and one elected lane issues: the
+// instruction takes its descriptors from uniform registers, and only in
+// warp-uniform code with uniform operands does the compiler keep them there.  A
+// loop of one lane (lane == 0) issued an MMA every 146 cycles whatever its size;
+// this form, unrolled, with the accumulate flag a constant, issues at the
+// tensor core's own pace: 128 cycles for 128 x 256 x 16, 64 for 128 x 128, 48 for
+// 128 x 64 (operand reads from shared memory), 40 for less.
+// (elect.sync picks the same lane each time, so the commits below cover the
+// MMAs issued here.)  All lanes of the warp call these.
+template <bool ACC>
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc) {
   asm volatile(
-      "{ .reg .pred p; setp.ne.b32 p, %4, 0; "
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(tmem),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
+      "{ .reg .pred p, e; elect.sync _|e, 0xffffffff; setp.ne.b32 p, %4, 0; "
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(tmem),
+      "l"(ad), "l"(bd), "r"(idesc), "n"(ACC ? 1 : 0)
       : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+      "{ .reg .pred e; elect.sync _|e, 0xffffffff; "
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0]; }" ::"r"(
           su32(mbar))
       : "memory");
 }
+
+// a value that is the same in every lane, in a form the compiler knows to be
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 __device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(b)), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t *b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_n(uint64_t *b, uint32_t n) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(n) : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *b, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes)
@@ -79,6 +96,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity,
     if (!done && (it > kMbarSpin || (stop && (it & 255) == 255 && *stop))) return false;
   }
   return true;
+}
+
+// the same by every lane of a warp, with one answer
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *mbar, uint32_t parity,
+                                               const volatile int *stop = nullptr) {
+  return __all_sync(0xffffffffu, mbar_wait(mbar, parity, stop));
 }
 
 // bulk asynchronous copy global -> shared, completing `bytes` on the mbarrier
