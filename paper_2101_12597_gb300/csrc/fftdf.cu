@@ -27,7 +27,11 @@ namespace etdm {
 
 constexpr int kDfThreads = 256;
 constexpr int kZPairs = 8;    // line pairs per block of the z passes
-constexpr int kXYLines = 8;   // lines per block of the x and y passes (4 blocks per SM)
+
+// Lines per block of the x and y passes (4 blocks per SM): a radix-4 stage has
+// lines n / 4 butterflies for 256 threads, so 8 lines from n = 80 up and 16
+// below (n = 48: 96 of the threads had work with 8).
+__host__ __device__ __forceinline__ int xy_lines(int n) { return n >= 80 ? 8 : 16; }
 
 // ---- float-pair scalars (hi, lo) and complex numbers ---------------------------
 struct dcx {
@@ -113,7 +117,7 @@ __device__ void df_stage(const float4 *in, float4 *out, int n, int Ns, int lines
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       dcx x = cx_ld(src[j + r * nb]);
-      if (r > 0 && k > 0) x = cx_mul(x, tw_get(tw, (r * k * step) % n, sign));
+      if (r > 0 && k > 0) x = cx_mul(x, tw_get(tw, r * k * step, sign));  // r k step < n
       v[r] = x;
     }
     if (R == 2) {
@@ -146,6 +150,36 @@ __device__ void df_stage(const float4 *in, float4 *out, int n, int Ns, int lines
   }
 }
 
+// A stage of a large radix, a thread per output: the same operations in the
+// same order as a butterfly of df_stage would do for that output, with its R
+// inputs' twiddle products done again by each of the R threads.  One thread
+// per radix-11 butterfly ran some 6000 dependent operations out of local
+// memory, with a handful of threads of a block at work (z passes of a 36 x 28 x
+// 44 grid: 50 us).
+template <int R>
+__device__ void df_stage_out(const float4 *in, float4 *out, int n, int Ns, int lines, const float4 *tw,
+                             int sign) {
+  const int nb = n / R;
+  const int step = n / (Ns * R);
+  for (int e = threadIdx.x; e < lines * n; e += blockDim.x) {
+    const int l = e / n, o = e % n;
+    const int w = o % (Ns * R), qq = w / Ns, k = w % Ns;
+    const float4 *src = in + (long)l * n + o / (Ns * R) * Ns + k;
+    dcx acc = cx_ld(src[0]);
+    int t0 = 0, t1 = 0;  // r k step mod n, r qq mod R
+    for (int r = 1; r < R; ++r) {
+      t0 += k * step;
+      if (t0 >= n) t0 -= n;
+      t1 += qq;
+      if (t1 >= R) t1 -= R;
+      dcx x = cx_ld(src[r * nb]);
+      if (k > 0) x = cx_mul(x, tw_get(tw, t0, sign));
+      acc = cx_add(acc, cx_mul(x, tw_get(tw, t1 * nb, sign)));
+    }
+    out[(long)l * n + o] = cx_st(acc);
+  }
+}
+
 // In-place (ping-pong) transform of `lines` lines held in b0; returns the buffer
 // holding the result.  Ends with a block barrier.  BIG: radices 7, 11, 13 are
 // compiled in (only grids with those factors need them; they cost registers).
@@ -163,9 +197,9 @@ __device__ float4 *df_fft(float4 *b0, float4 *b1, const DfPlan &pl, int lines, c
       case 5: df_stage<5>(in, out, pl.n, Ns, lines, tw, sign); break;
       default:
         if constexpr (BIG) {
-          if (R == 7) df_stage<7>(in, out, pl.n, Ns, lines, tw, sign);
-          else if (R == 11) df_stage<11>(in, out, pl.n, Ns, lines, tw, sign);
-          else df_stage<13>(in, out, pl.n, Ns, lines, tw, sign);
+          if (R == 7) df_stage_out<7>(in, out, pl.n, Ns, lines, tw, sign);
+          else if (R == 11) df_stage_out<11>(in, out, pl.n, Ns, lines, tw, sign);
+          else df_stage_out<13>(in, out, pl.n, Ns, lines, tw, sign);
         }
         break;
     }
@@ -226,15 +260,15 @@ __global__ void __launch_bounds__(kDfThreads, 4) yfft_kernel(const DfArgs *av, c
   extern __shared__ __align__(16) float4 ysm[];
   if (!active[blockIdx.y]) return;
   const DfArgs &a = av[blockIdx.y];
-  const int ny = a.ny, nzh = a.nzh;
+  const int ny = a.ny, nzh = a.nzh, kl = xy_lines(ny);
   const long nlines = (long)a.nx * nzh;
-  const long q0 = (long)blockIdx.x * kXYLines;
+  const long q0 = (long)blockIdx.x * kl;
   if (q0 >= nlines) return;
-  float4 *tw = ysm, *b0 = ysm + ny, *b1 = b0 + kXYLines * ny;
+  float4 *tw = ysm, *b0 = ysm + ny, *b1 = b0 + kl * ny;
   load_tw(tw, a.twy, ny);
-  const int lines = (int)min((long)kXYLines, nlines - q0);
-  for (int q = threadIdx.x; q < kXYLines * ny; q += blockDim.x) {
-    const int y = q / kXYLines, l = q % kXYLines;
+  const int lines = (int)min((long)kl, nlines - q0);
+  for (int q = threadIdx.x; q < kl * ny; q += blockDim.x) {
+    const int y = q / kl, l = q % kl;
     if (l < lines) {
       const long line = q0 + l, x = line / nzh, kz = line % nzh;
       b0[l * ny + y] = a.H[(x * ny + y) * nzh + kz];
@@ -242,8 +276,8 @@ __global__ void __launch_bounds__(kDfThreads, 4) yfft_kernel(const DfArgs *av, c
   }
   __syncthreads();
   const float4 *Y = df_fft<BIG>(b0, b1, a.py, lines, tw, sign);
-  for (int q = threadIdx.x; q < kXYLines * ny; q += blockDim.x) {
-    const int y = q / kXYLines, l = q % kXYLines;
+  for (int q = threadIdx.x; q < kl * ny; q += blockDim.x) {
+    const int y = q / kl, l = q % kl;
     if (l < lines) {
       const long line = q0 + l, x = line / nzh, kz = line % nzh;
       a.H[(x * ny + y) * nzh + kz] = Y[l * ny + y];
@@ -257,22 +291,22 @@ __global__ void __launch_bounds__(kDfThreads, 4) xpois_kernel(const DfArgs *av, 
   extern __shared__ __align__(16) float4 xsm[];
   if (!active[blockIdx.y]) return;
   const DfArgs &a = av[blockIdx.y];
-  const int nx = a.nx, ny = a.ny, nzh = a.nzh;
+  const int nx = a.nx, ny = a.ny, nzh = a.nzh, kl = xy_lines(nx);
   const long nlines = (long)ny * nzh;
-  const long q0 = (long)blockIdx.x * kXYLines;
+  const long q0 = (long)blockIdx.x * kl;
   if (q0 >= nlines) return;
-  float4 *tw = xsm, *b0 = xsm + nx, *b1 = b0 + kXYLines * nx;
+  float4 *tw = xsm, *b0 = xsm + nx, *b1 = b0 + kl * nx;
   load_tw(tw, a.twx, nx);
-  const int lines = (int)min((long)kXYLines, nlines - q0);
+  const int lines = (int)min((long)kl, nlines - q0);
   const long stride = (long)ny * nzh;
-  for (int q = threadIdx.x; q < kXYLines * nx; q += blockDim.x) {
-    const int x = q / kXYLines, l = q % kXYLines;
+  for (int q = threadIdx.x; q < kl * nx; q += blockDim.x) {
+    const int x = q / kl, l = q % kl;
     if (l < lines) b0[l * nx + x] = a.H[x * stride + q0 + l];
   }
   __syncthreads();
   float4 *Xf = df_fft<BIG>(b0, b1, a.px, lines, tw, -1);
-  for (int q = threadIdx.x; q < kXYLines * nx; q += blockDim.x) {
-    const int x = q / kXYLines, l = q % kXYLines;
+  for (int q = threadIdx.x; q < kl * nx; q += blockDim.x) {
+    const int x = q / kl, l = q % kl;
     if (l < lines) {
       const float2 kp = a.kpois[x * stride + q0 + l];
       const dcx v = cx_ld(Xf[l * nx + x]);
@@ -282,8 +316,8 @@ __global__ void __launch_bounds__(kDfThreads, 4) xpois_kernel(const DfArgs *av, 
   __syncthreads();
   float4 *other = Xf == b0 ? b1 : b0;
   const float4 *Xi = df_fft<BIG>(Xf, other, a.px, lines, tw, +1);
-  for (int q = threadIdx.x; q < kXYLines * nx; q += blockDim.x) {
-    const int x = q / kXYLines, l = q % kXYLines;
+  for (int q = threadIdx.x; q < kl * nx; q += blockDim.x) {
+    const int x = q / kl, l = q % kl;
     if (l < lines) a.H[x * stride + q0 + l] = Xi[l * nx + x];
   }
 }
@@ -480,11 +514,11 @@ DfLaunch df_launch_plan(const std::vector<DfArgs> &args) {
   DfLaunch L{};
   for (const DfArgs &a : args) {
     L.zb = std::max(L.zb, (int)(((long)a.nx * a.ny + 2 * kZPairs - 1) / (2 * kZPairs)));
-    L.yb = std::max(L.yb, (int)(((long)a.nx * a.nzh + kXYLines - 1) / kXYLines));
-    L.xb = std::max(L.xb, (int)(((long)a.ny * a.nzh + kXYLines - 1) / kXYLines));
+    L.yb = std::max(L.yb, (int)(((long)a.nx * a.nzh + xy_lines(a.ny) - 1) / xy_lines(a.ny)));
+    L.xb = std::max(L.xb, (int)(((long)a.ny * a.nzh + xy_lines(a.nx) - 1) / xy_lines(a.nx)));
     L.smz = std::max(L.smz, (size_t)(a.nz + 2 * kZPairs * a.nz) * sizeof(float4));
-    L.smy = std::max(L.smy, (size_t)(a.ny + 2 * kXYLines * a.ny) * sizeof(float4));
-    L.smx = std::max(L.smx, (size_t)(a.nx + 2 * kXYLines * a.nx) * sizeof(float4));
+    L.smy = std::max(L.smy, (size_t)(a.ny + 2 * xy_lines(a.ny) * a.ny) * sizeof(float4));
+    L.smx = std::max(L.smx, (size_t)(a.nx + 2 * xy_lines(a.nx) * a.nx) * sizeof(float4));
     for (const DfPlan *p : {&a.px, &a.py, &a.pz})
       for (int i = 0; i < p->nst; ++i) L.big = L.big || p->radix[i] > 5;
   }
