@@ -49,9 +49,11 @@ cudaError_t launch_oz_zgemm(const OzWork &W, const double2 *A, int opa, const do
 size_t heev_work_bytes(int n, int batch);
 // method 0: implicit QL on the tridiagonal (robust for any spectrum; used at
 // set-up); 1: bisection and inverse iteration (parallel over the eigenvalues;
-// used for iA(k) in every evaluation)
+// used for iA(k) in every evaluation).  oz: back-transformation in blocks of
+// reflectors on the tensor cores (their workspace; null: reflector by reflector)
 cudaError_t launch_heev(double2 *A, double *w, double2 *V, int n, int batch, void *work,
-                        int *flags, cudaStream_t s, int method = 0);
+                        int *flags, cudaStream_t s, int method = 0, const OzWork *oz = nullptr);
+int heev_launches(int n, const OzWork *oz);  // kernels of one call with method 1
 
 
 }  // namespace etdm
