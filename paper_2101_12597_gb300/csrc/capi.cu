@@ -89,20 +89,15 @@ void evaluate(etdm_handle *h, const double *a, double *E, double *g, cudaStream_
       CUDA_TRY(launch_mixed_potential(h->plan, s));
       h->n_gridpart = df_pot_blocks(h);
     } else {
-      CUDA_TRY(launch_pack_real(h, h->d_rho, h->d_fft, s));
-      CUDA_TRY(fft3d(h, h->d_fft, -1, s));
-      CUDA_TRY(launch_poisson_scale(h, h->d_fft, s));
-      CUDA_TRY(fft3d(h, h->d_fft, +1, s));
-      CUDA_TRY(launch_potential(h, s));
-      h->n_gridpart = kPotBlocks;
+      CUDA_TRY(launch_potential(h, h->d_rho, h->d_vtot, h->d_gridpart, false, 0.0, s));
+      h->n_gridpart = pot_blocks(h);
     }
     t.done();
   }
-  // kernels: dense forward and reverse; mixed: O slices (column maxima, then
-  // the slices), density, 5 potential passes, V and its fixed-point
-  // conversion; FP64: density, pack, 2 x 3 FFT passes, scale, potential (+ V
-  // with the gradient)
-  h->launches += 12;
+  // kernels: dense forward and reverse, 5 potential passes; mixed: O slices
+  // (column maxima, then the slices), density, V and its fixed-point
+  // conversion; FP64: density (+ V with the gradient)
+  h->launches += 7 + (mixed ? 5 : rho64_launches(h));
   if (mixed) {  // also needed for the energy: first-order correction of D's quantization
     StageTimer t(h, s, ETDM_STAGE_VMAT);
     CUDA_TRY(launch_mixed_vmat(h->plan, s));
@@ -111,7 +106,7 @@ void evaluate(etdm_handle *h, const double *a, double *E, double *g, cudaStream_
     StageTimer t(h, s, ETDM_STAGE_VMAT);
     CUDA_TRY(launch_vmat_fp64(h, h->d_vtot, h->d_H, s));
     t.done();
-    h->launches += 1;
+    h->launches += vmat64_launches(h);
   }
   {
     StageTimer t(h, s, ETDM_STAGE_DENSE_REV);
@@ -587,8 +582,10 @@ void init_impl(etdm_handle *h, const etdm_system *sys, const etdm_options *opt) 
   h->d_vtot = dalloc<double>(h, h->G);
   h->d_fft = dalloc<double2>(h, h->G);
   h->d_tw = dalloc<double2>(h, h->n[0] + h->n[1] + h->n[2]);
-  h->n_gridpart = kPotBlocks;
-  h->d_gridpart = dalloc<double>(h, 3 * std::max(kPotBlocks, df_pot_blocks(h)));
+  h->n_gridpart = pot_blocks(h);
+  h->d_gridpart = dalloc<double>(h, 3 * std::max(pot_blocks(h), df_pot_blocks(h)));
+  h->d_kpois64 = dalloc<double>(h, (size_t)h->n[0] * h->n[1] * (h->n[2] / 2 + 1));
+  CUDA_TRY(launch_potential_setup(h, s));
   CUDA_TRY(launch_twiddles(h, s));
   CUDA_TRY(launch_vext_recip(h, s));
   CUDA_TRY(fft3d(h, h->d_fft, +1, s));

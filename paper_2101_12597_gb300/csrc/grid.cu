@@ -533,7 +533,7 @@ cudaError_t launch_rho_k(etdm_handle *h, const double *DR, double *rho, cudaStre
   return cudaGetLastError();
 }
 
-// VR[R][mu_a][mu_b] += dV sum_p X_ap v_p X_bp for every ordered pair of list
+// VR[R][mu_a][mu_b] (zeroed by the launcher) += dV sum_p X_ap v_p X_bp for every ordered pair of list
 // entries (computed once per unordered pair).
 __global__ void __launch_bounds__(kRhoThreads) vmat_k_kernel(GridGeom g, Tables tb,
                                                              const int *tile_ptr,
@@ -599,7 +599,9 @@ __global__ void __launch_bounds__(kRhoThreads) vmat_k_kernel(GridGeom g, Tables 
 
 cudaError_t launch_vmat_k(etdm_handle *h, const double *v, double *VR, cudaStream_t s) {
   size_t sm = (size_t)h->max_list * (kTP + 1) * 16 + (size_t)h->max_list * 8 + 16;
-  cudaError_t e = cudaFuncSetAttribute(vmat_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaMemsetAsync(VR, 0, (size_t)h->kg.nR * h->M * h->M * 8, s);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(vmat_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   vmat_k_kernel<<<h->n_tiles, kRhoThreads, sm, s>>>(h->geom, tables_of(h), h->d_tile_ptr,

@@ -18,7 +18,6 @@ constexpr int kImgN = 2 * kImgMax + 1;
 constexpr int kTaylor = 10;         // Taylor terms of cos sqrt(Q), sin sqrt(Q)/sqrt(Q)
 constexpr int kJmax = 8;            // doublings: |P|_F <= 4^8
 constexpr int kMaxList = 200;       // max truncation-list length per tile (FP64 path)
-constexpr int kPotBlocks = 512;     // blocks (and energy partials) of the potential pass
 constexpr int kMaxFFT = 256;        // max grid points per axis
 constexpr long kSpinLimit = 2000000;   // bounded device waits (a few seconds at most)
 
@@ -416,6 +415,7 @@ struct etdm_handle {
   // grid
   double *d_vext = nullptr, *d_rho = nullptr, *d_vtot = nullptr;
   double2 *d_fft = nullptr;
+  double *d_kpois64 = nullptr;  // [nx][ny][nz/2+1] Poisson kernel, FP64
   double2 *d_tw = nullptr;   // twiddles per axis (n[0]+n[1]+n[2])
   double *d_gridpart = nullptr;
   int n_gridpart = 0;
@@ -480,6 +480,9 @@ cudaError_t launch_scan(const int *d_in, long long *d_out, long n, long long *d_
                         cudaStream_t s);
 cudaError_t launch_npt2(etdm_handle *h, unsigned long long *d_sum, cudaStream_t s);
 cudaError_t launch_overlap_kinetic(etdm_handle *h, cudaStream_t s);
+// kernels of one density or potential-matrix pass of the FP64 arithmetic
+inline int rho64_launches(const etdm_handle *) { return 1; }
+inline int vmat64_launches(const etdm_handle *) { return 1; }
 cudaError_t launch_rho_fp64(etdm_handle *h, const double *D, double *rho, cudaStream_t s);
 cudaError_t launch_vmat_fp64(etdm_handle *h, const double *v, double *Hacc, cudaStream_t s);
 // fft and potential (potential.cu)
@@ -487,9 +490,12 @@ cudaError_t launch_twiddles(etdm_handle *h, cudaStream_t s);
 cudaError_t fft3d(etdm_handle *h, double2 *data, int sign, cudaStream_t s);
 cudaError_t launch_vext_recip(etdm_handle *h, cudaStream_t s);
 cudaError_t launch_real_part(etdm_handle *h, const double2 *src, double *dst, cudaStream_t s);
-cudaError_t launch_pack_real(etdm_handle *h, const double *src, double2 *dst, cudaStream_t s);
-cudaError_t launch_poisson_scale(etdm_handle *h, double2 *data, cudaStream_t s);
-cudaError_t launch_potential(etdm_handle *h, cudaStream_t s);
+cudaError_t launch_potential_setup(etdm_handle *h, cudaStream_t s);  // Poisson kernel table
+// v and the energy partials (3 per block) of rho; sic: an orbital density's
+// potential and one partial per block, times -fk
+cudaError_t launch_potential(etdm_handle *h, const double *rho, double *v, double *part, bool sic,
+                             double fk, cudaStream_t s);
+int pot_blocks(const etdm_handle *h);
 // dense (dense.cu)
 cudaError_t launch_gemm(const Phase &ph, cudaStream_t s);
 cudaError_t launch_dense_forward(etdm_handle *h, const double *a, cudaStream_t s);

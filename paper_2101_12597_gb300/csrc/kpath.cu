@@ -38,7 +38,11 @@ void check_device_status(etdm_handle *h, cudaStream_t s, const char *where) {
 // the handle has their workspace (oz_takes), else FP64 FMA
 cudaError_t prod_k(etdm_handle *h, const double2 *A, int opa, const double2 *B, int opb, double2 *C,
                    cudaStream_t s, double alpha = 1.0, double beta = 0.0) {
-  if (h->oz.n == h->M) return launch_oz_zgemm(h->oz, A, opa, B, opb, C, h->nk, alpha, beta, h->d_flags, s);
+  if (h->oz.n == h->M) {
+    h->launches += 3L * ((h->nk + h->oz.group - 1) / h->oz.group);
+    return launch_oz_zgemm(h->oz, A, opa, B, opb, C, h->nk, alpha, beta, h->d_flags, s);
+  }
+  h->launches += 1;
   return zgemm_sq(A, opa, B, opb, C, h->M, h->nk, s, alpha, beta);
 }
 
@@ -87,7 +91,7 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
     h->d_sicX = dalloc<double2>(h, M);
     h->d_sicn = dalloc<double>(h, h->G);
     h->d_sicv = dalloc<double>(h, h->G);
-    h->d_sicpart = dalloc<double>(h, (size_t)std::max(h->N, 1) * k_sic_parts());
+    h->d_sicpart = dalloc<double>(h, (size_t)std::max(h->N, 1) * pot_blocks(h));
   }
   if (h->kexpm == ETDM_EXPM_SS) {
     for (double2 **p : {&h->d_kB, &h->d_kB2, &h->d_kB3}) *p = dalloc<double2>(h, KM);
@@ -99,7 +103,6 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
 
   // S(k), T(k); h_core(k) = T(k) + V_ext(k)
   CUDA_TRY(k_overlap_kinetic(h, s));
-  CUDA_TRY(cudaMemsetAsync(h->d_kVR, 0, (size_t)G.nR * MM * 8, s));
   CUDA_TRY(launch_vmat_k(h, h->d_vext, h->d_kVR, s));
   CUDA_TRY(k_hamiltonian(G, h->d_kT, h->d_kVR, h->d_kH, s));
   CUDA_TRY(k_hermitize(h->d_kH, nk, M, s));
@@ -168,7 +171,7 @@ void expm_ss_k(etdm_handle *h, const double *a, double2 *U, cudaStream_t s) {
     std::swap(Y, Yn);
   }
   CUDA_TRY(cudaMemcpyAsync(U, Y, (size_t)nk * M * M * 16, cudaMemcpyDeviceToDevice, s));
-  h->launches += 17 + (sq > 0 ? 1 : 0) + sq;
+  h->launches += 9 + (sq > 0 ? 1 : 0);  // A, its norm, the coefficients
 }
 
 }  // namespace
@@ -186,13 +189,8 @@ void sic_orbitals_k(etdm_handle *h, cudaStream_t s) {
     CUDA_TRY(k_rank1(h->d_kO, k, M, h->d_sicD, s));
     CUDA_TRY(k_dr(G, h->d_sicD, h->d_kDR, s));
     CUDA_TRY(launch_rho_k(h, h->d_kDR, h->d_sicn, s));
-    CUDA_TRY(launch_pack_real(h, h->d_sicn, h->d_fft, s));
-    CUDA_TRY(fft3d(h, h->d_fft, -1, s));
-    CUDA_TRY(launch_poisson_scale(h, h->d_fft, s));
-    CUDA_TRY(fft3d(h, h->d_fft, +1, s));
-    CUDA_TRY(k_sic_potential(h->d_sicn, h->d_fft, h->d_sicv, h->G, h->dV, fk,
-                             h->d_sicpart + (size_t)k * k_sic_parts(), s));
-    CUDA_TRY(cudaMemsetAsync(h->d_kVR, 0, (size_t)G.nR * M * M * 8, s));
+    CUDA_TRY(launch_potential(h, h->d_sicn, h->d_sicv, h->d_sicpart + (size_t)k * pot_blocks(h), true,
+                              fk, s));
     CUDA_TRY(launch_vmat_k(h, h->d_sicv, h->d_kVR, s));
     CUDA_TRY(k_hamiltonian(G, nullptr, h->d_kVR, h->d_sicV, s));
     ZgemmArgs x{};  // X = V^k O_k
@@ -206,7 +204,8 @@ void sic_orbitals_k(etdm_handle *h, cudaStream_t s) {
     y.opa = 1; y.opb = 0; y.alpha = make_double2(1.0, 0.0); y.beta = make_double2(0.0, 0.0);
     CUDA_TRY(launch_zgemm(y, 1, s));
   }
-  h->launches += 16L * h->N;
+  // rank-1 D, DR, density, 5 potential passes, V, H, 2 products
+  h->launches += (long)h->N * (10 + rho64_launches(h) + vmat64_launches(h));
 }
 
 void refresh_reference_k(etdm_handle *h, cudaStream_t s) {
@@ -247,7 +246,7 @@ void commutator_norms_k(etdm_handle *h, const double *a, const double *g, double
   }
   *nL = sqrt(l2);
   *nC = sqrt(c2);
-  h->launches += 6;
+  h->launches += 4;
 }
 
 void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStream_t s) {
@@ -283,19 +282,16 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   CUDA_TRY(launch_rho_k(h, h->d_kDR, h->d_rho, s));
   tr.done();
   StageTimer tp(h, s, ETDM_STAGE_POTENTIAL);
-  CUDA_TRY(launch_pack_real(h, h->d_rho, h->d_fft, s));
-  CUDA_TRY(fft3d(h, h->d_fft, -1, s));
-  CUDA_TRY(launch_poisson_scale(h, h->d_fft, s));
-  CUDA_TRY(fft3d(h, h->d_fft, +1, s));
-  CUDA_TRY(launch_potential(h, s));
-  h->n_gridpart = kPotBlocks;
+  CUDA_TRY(launch_potential(h, h->d_rho, h->d_vtot, h->d_gridpart, false, 0.0, s));
+  h->n_gridpart = pot_blocks(h);
   if (h->sic) sic_orbitals_k(h, s);
   tp.done();
   StageTimer tk(h, s, ETDM_STAGE_DENSE_REV);
   CUDA_TRY(k_energy(h->d_kD, h->d_kT, KM, h->d_kpart, h->d_gridpart, h->n_gridpart, h->d_eterms,
                     E, h->d_flags, s, h->sic ? h->d_sicpart : nullptr,
-                    h->sic ? h->N * k_sic_parts() : 0));
-  h->launches += 25;
+                    h->sic ? h->N * pot_blocks(h) : 0));
+  // exp: iA, the eigensolver and the phases (eig); O f, DR, density, 5 potential passes, 2 energy sums
+  h->launches += (ss ? 0 : 2 + heev_launches(M, &h->oz)) + 9 + rho64_launches(h);
   if (!g) {
     tk.done();
     return;
@@ -303,7 +299,6 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   tk.done();
   // H(k), L = [F, O^dagger H O], and the Eq. 39 adjoint
   StageTimer tv(h, s, ETDM_STAGE_VMAT);
-  CUDA_TRY(cudaMemsetAsync(h->d_kVR, 0, (size_t)G.nR * M * M * 8, s));
   CUDA_TRY(launch_vmat_k(h, h->d_vtot, h->d_kVR, s));
   tv.done();
   StageTimer tg(h, s, ETDM_STAGE_DENSE_REV);
@@ -315,7 +310,7 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   if (ss) {  // Eq. 42: G ~ L^T
     CUDA_TRY(k_grad_vars(h->d_kX2, g, nk, M, s));
     tg.done();
-    h->launches += 5;
+    h->launches += 3 + h->sic + vmat64_launches(h);
     return;
   }
   CUDA_TRY(prod_k(h, h->d_kX2, 0, h->d_kW, 0, h->d_kX1, s));    // L W
@@ -325,7 +320,7 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kW, 1, h->d_kX2, s));    // G^T
   CUDA_TRY(k_grad_vars(h->d_kX2, g, nk, M, s));
   tg.done();
-  h->launches += 11;
+  h->launches += 4 + h->sic + vmat64_launches(h);
 }
 
 }  // namespace etdm

@@ -87,9 +87,6 @@ cudaError_t k_energy(const double2 *D, const double2 *T, long n, double *part,
 // PZ-SIC (Gamma point): orbital density matrix, orbital potential and energy
 // partials, the L correction
 cudaError_t k_rank1(const double2 *O, int k, int M, double2 *D, cudaStream_t s);
-int k_sic_parts();
-cudaError_t k_sic_potential(const double *n, const double2 *vh, double *v, long G, double dV,
-                            double fk, double *part, cudaStream_t s);
 cudaError_t k_sic_L(double2 *L, const double2 *S, const double *f, int M, cudaStream_t s);
 cudaError_t k_occupation(const double *eps, const double *kw, int nk, int M, double ne, double kT,
                          double *f, double *mu, cudaStream_t s);
