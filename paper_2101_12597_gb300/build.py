@@ -15,7 +15,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libetdm.so")
 SOURCES = ["capi.cu", "dense.cu", "grid.cu", "potential.cu", "mixed.cu", "fftdf.cu", "noalloc.cu",
            "plan.cu", "batch.cu", "kpoint.cu", "kpath.cu",
-           "ozgemm.cu"]
+           "ozgemm.cu", "ozgrid.cu"]
 HEADERS = ["internal.h", "device.cuh", "host.h", "pair.cuh", "linesearch.h", "tc.cuh", "kpoint.h",
            "ozdigits.cuh", "tcgemm.cuh"]
 NVCC = os.environ.get("NVCC", "nvcc")

@@ -377,6 +377,19 @@ void etdm::build_vgroups(etdm_handle *h, int vg_max, cudaStream_t s) {
   CUDA_TRY(launch_xv_build(h, s));
 }
 
+void etdm::setup_ox(etdm_handle *h, bool images, cudaStream_t s) {
+  int T = 0, max_list = 0, *d_ptr = nullptr, *d_keys = nullptr;
+  long n = 0;
+  const GridGeom geom = make_geom(h, 4, 4, 8, &T);
+  build_lists(h, geom, T, &d_ptr, &d_keys, &n, &max_list, INT32_MAX, s);
+  std::vector<int> ptr(T + 1), keys(n);
+  CUDA_TRY(cudaMemcpy(ptr.data(), d_ptr, (T + 1) * sizeof(int), cudaMemcpyDeviceToHost));
+  if (n > 0) CUDA_TRY(cudaMemcpy(keys.data(), d_keys, n * sizeof(int), cudaMemcpyDeviceToHost));
+  ox_setup(h, geom, T, ptr, keys, d_keys, images, s);
+  dfree(h, d_ptr);
+  dfree(h, d_keys);
+}
+
 // L-BFGS memory, line-search buffers and reduction scratch for h->nvar
 // variables (both parametrizations).
 void etdm::alloc_opt_buffers(etdm_handle *h) {
@@ -591,6 +604,7 @@ void init_impl(etdm_handle *h, const etdm_system *sys, const etdm_options *opt) 
   CUDA_TRY(fft3d(h, h->d_fft, +1, s));
   CUDA_TRY(launch_real_part(h, h->d_fft, h->d_vext, s));
   if (h->precision == ETDM_PREC_MIXED) CUDA_TRY(launch_df_setup(h, s));  // twiddles, v_ext, Poisson kernel
+  if (h->precision == ETDM_PREC_FP64 && !h->kpath) setup_ox(h, false, s);
   if (h->kpath) {  // full A over k-points: its own matrices and reference
     h->d_E = dalloc<double>(h, 2);
     h->d_eterms = dalloc<double>(h, 4);

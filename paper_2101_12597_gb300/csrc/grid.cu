@@ -380,6 +380,7 @@ static size_t rho_smem(int n) {
 }
 
 cudaError_t launch_rho_fp64(etdm_handle *h, const double *D, double *rho, cudaStream_t s) {
+  if (h->ox.n_tiles) return launch_ox_rho(h, D, rho, s);
   size_t sm = rho_smem(h->max_list);
   cudaError_t e = cudaFuncSetAttribute(rho_fp64_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -449,6 +450,7 @@ __global__ void __launch_bounds__(kRhoThreads) vmat_fp64_kernel(GridGeom g, Tabl
 }
 
 cudaError_t launch_vmat_fp64(etdm_handle *h, const double *v, double *Hacc, cudaStream_t s) {
+  if (h->ox.n_tiles) return launch_ox_vmat(h, v, Hacc, s);
   size_t sm = (size_t)h->max_list * (kTP + 1) * 16 + (size_t)h->max_list * 4 + 16;
   cudaError_t e = cudaFuncSetAttribute(vmat_fp64_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -524,6 +526,7 @@ __global__ void __launch_bounds__(kRhoThreads) rho_k_kernel(GridGeom g, Tables t
 }
 
 cudaError_t launch_rho_k(etdm_handle *h, const double *DR, double *rho, cudaStream_t s) {
+  if (h->ox.n_tiles) return launch_ox_rho(h, DR, rho, s);
   size_t sm = rho_smem(h->max_list) + (size_t)h->max_list * 4;
   cudaError_t e = cudaFuncSetAttribute(rho_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
@@ -598,6 +601,7 @@ __global__ void __launch_bounds__(kRhoThreads) vmat_k_kernel(GridGeom g, Tables 
 }
 
 cudaError_t launch_vmat_k(etdm_handle *h, const double *v, double *VR, cudaStream_t s) {
+  if (h->ox.n_tiles) return launch_ox_vmat_k(h, v, VR, s);
   size_t sm = (size_t)h->max_list * (kTP + 1) * 16 + (size_t)h->max_list * 8 + 16;
   cudaError_t e = cudaMemsetAsync(VR, 0, (size_t)h->kg.nR * h->M * h->M * 8, s);
   if (e != cudaSuccess) return e;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <string>
+#include <vector>
 
 #include "internal.h"
 
@@ -93,6 +94,12 @@ struct StageTimer {
 
 // V groups of at most vg_max tiles, their tables and X^T slices (capi.cu)
 void build_vgroups(etdm_handle *h, int vg_max, cudaStream_t s);
+
+// Tables of the FP64 grid passes on the tensor cores: setup_ox (capi.cu) builds
+// the 4 x 4 x 8 tiles' image lists, ox_setup (ozgrid.cu) the rest
+void setup_ox(etdm_handle *h, bool images, cudaStream_t s);
+void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vector<int> &kptr,
+              const std::vector<int> &keys, const int *d_keys, bool images, cudaStream_t s);
 
 // L-BFGS memory, line-search buffers and reduction scratch for h->nvar
 // variables (capi.cu).

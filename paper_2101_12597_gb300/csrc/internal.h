@@ -290,6 +290,20 @@ struct OzWork {
   int *rexp = nullptr, *cexp = nullptr;
 };
 
+// Tables of the FP64 grid passes on the tensor cores (ozgrid.cu; n_tiles = 0:
+// none, the passes of grid.cu run).
+struct OxGrid {
+  GridGeom geom{};
+  int n_tiles = 0;
+  bool images = false;          // entries are images (k-points), else functions
+  int bX = 0, hexp = 0;         // exponents of X and of V's fixed point
+  int *ptr = nullptr, *id = nullptr;
+  long long *x = nullptr, *vt = nullptr, *dfix = nullptr;
+  unsigned long long *V = nullptr;
+  signed char *rsh = nullptr;
+  int *part = nullptr, *bexp = nullptr, *ee = nullptr, *ct = nullptr;
+};
+
 }  // namespace etdm
 
 struct etdm_handle {
@@ -319,6 +333,7 @@ struct etdm_handle {
   double *d_kDR = nullptr, *d_kVR = nullptr;  // [nR][M][M]
   void *d_kwork = nullptr;      // eigensolver workspace
   etdm::OzWork oz{};            // tensor-core products (large M)
+  etdm::OxGrid ox{};            // FP64 grid passes on the tensor cores
   bool kref_set = false;        // reference given by etdm_set_reference
   int kexpm = 0;                // ETDM_EXPM_EIG (Eq. 35, Eq. 39) or ETDM_EXPM_SS (Eq. 38, Eq. 42)
   int tri_method = 1;           // tridiagonal eigenpairs of iA(k): 1 bisection + inverse iteration, 0 QL
@@ -481,10 +496,15 @@ cudaError_t launch_scan(const int *d_in, long long *d_out, long n, long long *d_
 cudaError_t launch_npt2(etdm_handle *h, unsigned long long *d_sum, cudaStream_t s);
 cudaError_t launch_overlap_kinetic(etdm_handle *h, cudaStream_t s);
 // kernels of one density or potential-matrix pass of the FP64 arithmetic
-inline int rho64_launches(const etdm_handle *) { return 1; }
-inline int vmat64_launches(const etdm_handle *) { return 1; }
+inline int rho64_launches(const etdm_handle *h) { return h->ox.n_tiles ? 2 : 1; }
+inline int vmat64_launches(const etdm_handle *h) { return h->ox.n_tiles ? 4 : 1; }
 cudaError_t launch_rho_fp64(etdm_handle *h, const double *D, double *rho, cudaStream_t s);
 cudaError_t launch_vmat_fp64(etdm_handle *h, const double *v, double *Hacc, cudaStream_t s);
+// the same on the tensor cores (ozgrid.cu); the launchers above take them
+// when the handle has their tables
+cudaError_t launch_ox_rho(etdm_handle *h, const double *D, double *rho, cudaStream_t s);
+cudaError_t launch_ox_vmat(etdm_handle *h, const double *v, double *H, cudaStream_t s);
+cudaError_t launch_ox_vmat_k(etdm_handle *h, const double *v, double *VR, cudaStream_t s);
 // fft and potential (potential.cu)
 cudaError_t launch_twiddles(etdm_handle *h, cudaStream_t s);
 cudaError_t fft3d(etdm_handle *h, double2 *data, int sign, cudaStream_t s);

@@ -1,0 +1,715 @@
+// FP64 grid passes on the 5th-generation tensor cores: basis -> grid density
+// (Eq. 2, 12) and grid -> basis potential matrix (Eq. 11) of the FP64 path and
+// of the full-A path, in exact base-256 digits (ozdigits.cuh).
+//
+// FP64 FMA bounds these passes on this part (1.05 TFLOP/s): the 4 x 4 x 4-tile
+// kernels of grid.cu take 11.2 ms (density) and 9.4 ms (V) for 96 atoms on a
+// 96^3 grid.  Here a 4 x 4 x 8 tile of 128 points with n <= 128 list entries is
+//   density:  Y = X D_loc (128 x n x n),  rho_p = sum_b Y_pb X_pb ,
+//   V:        V_loc = X^T (v X)           (n x n x 128),
+// with X, D and v in 64-bit fixed point and the products' digits on tcgen05;
+// sums stay exact in 64- and 128-bit integers up to rho (one rounding to FP64)
+// and to V's 64-bit fixed point, so no FP64 arithmetic is left in either pass
+// and V is independent of the order of its additions.
+//
+//   X: one entry per function and tile, periodic images of a function that
+//      reach the tile summed (the phase between images is 1 at the Gamma point;
+//      a box of 6.4 A has some 150 images of 16 functions per tile); with
+//      k-points one entry per image, the pair's lattice offset looked up.
+//      Evaluated once in FP64 at set-up and kept as fixed point, [entry][128].
+//   D: positive semidefinite, so |D_ab| <= sqrt(D_aa D_bb): D_ab 2^-(e_a + e_b)
+//      with D_aa < 2^2e_a in fixed point, and X_pa shifted by e_a in the density
+//      pass.  Where the density is faint because its functions' D is, it keeps
+//      its relative accuracy, which rho^(1/3) passes on to v (one power of two
+//      for all of D left 1e-9 of v, and 6e-11 of H, on an atom whose orbitals
+//      are empty).
+//   v: fixed point with the power of two of its largest element; 62 bits below
+//      it are nine more than FP64 keeps of it.
+//   V: 64-bit fixed point with a factor 2 in reserve over the Cauchy-Schwarz
+//      bound of |V_ab|, max |v dV| times the largest sum of X^2 of a function
+//      (sums wrap harmlessly in between).
+//
+// One persistent block per SM: warps 0-15 read the accumulators (lane quarter
+// w % 4, column quarter w / 4), warps 16-23 cut the digits of a K step of 16
+// into a four-stage ring, warp 24 issues the MMAs.  The columns of a tile go in
+// passes of 64 (eight orders of 64 columns fill tensor memory), the last one
+// 64, 32 or 16 wide.  A tile's K is at most 128, one exact chunk.
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "device.cuh"
+#include "host.h"
+#include "kpoint.h"
+#include "ozdigits.cuh"
+
+namespace etdm {
+
+constexpr int kOxP = 128;                       // points per tile (4 x 4 x 8)
+constexpr int kOxN = 128;                       // list entries per tile, at most
+constexpr int kOxCols = 64;                     // columns of a pass, at most
+constexpr int kOxA = kOzS * 128 * 32, kOxB = kOzS * kOxCols * 32;
+constexpr int kOxStage = kOxA + kOxB;           // 48 KB
+constexpr int kOxStages = 4;
+constexpr int kOxEpiW = 16, kOxBldW = 8;
+constexpr int kOxThreads = (kOxEpiW + kOxBldW + 1) * 32;
+constexpr int kOxParts = 256;                   // partial maxima of a fixed-point conversion
+
+struct OxArgs {
+  GridGeom g;               // 4 x 4 x 8 tiles
+  KGeom G;                  // lattice offsets (k-points)
+  int n_tiles, bX;          // |X| < 2^(bX - 1022)
+  const int *ptr, *id;      // entries of a tile; mu, or the image key (k-points)
+  const long long *x;       // [entry][128]
+  const signed char *rsh;   // [tile][128] left shift that fills a point's largest |X|
+  const long long *dfix;    // density: scaled D, or DR per offset
+  const int *ee, *ct;       // density: exponents e_a of the functions; -max e_a of a tile
+  const int *bexp;          // exponent field of v dV
+  double *rho;
+  const long long *vt;      // V: v dV in tile order
+  unsigned long long *V;    // V: sums, [M][M] (upper triangle), or [offset][M][M]
+  int sh;                   // V: left shift (right when negative) of a tile's sum
+  int full;                 // V: both triangles
+  int *flags;
+};
+
+__device__ __forceinline__ int ox_point(const GridGeom &g, int t, int p) {
+  const int bz = t % g.nbz, by = (t / g.nbz) % g.nby, bx = t / (g.nbz * g.nby);
+  const int i = bx * 4 + (p >> 5), j = by * 4 + ((p >> 3) & 3), k = bz * 8 + (p & 7);
+  return (i < g.nx && j < g.ny && k < g.nz) ? (i * g.ny + j) * g.nz + k : -1;
+}
+
+// index of the lattice offset n_a - n_b of two image keys, -1 beyond the table
+__device__ __forceinline__ int ox_ridx(const KGeom &G, int ka, int kb) {
+  const int rx = ((ka >> 6) & 7) - ((kb >> 6) & 7), ry = ((ka >> 3) & 7) - ((kb >> 3) & 7),
+            rz = (ka & 7) - (kb & 7);
+  if (abs(rx) > G.Rm[0] || abs(ry) > G.Rm[1] || abs(rz) > G.Rm[2]) return -1;
+  return ((rx + G.Rm[0]) * (2 * G.Rm[1] + 1) + ry + G.Rm[1]) * (2 * G.Rm[2] + 1) + rz + G.Rm[2];
+}
+
+// ---- set-up -------------------------------------------------------------------
+// X of a tile's entries in FP64 (into the fixed-point table's memory): entry e
+// sums the images keys[ek[e]] .. keys[ek[e + 1] - 1]
+__global__ void __launch_bounds__(kOxP) ox_basis_kernel(GridGeom g, Tables tb, const int *ptr,
+                                                        const int *ek, const int *keys, double *x) {
+  const int t = blockIdx.x, p = threadIdx.x;
+  const int bz = t % g.nbz, by = (t / g.nbz) % g.nby, bx = t / (g.nbz * g.nby);
+  const int i = bx * 4 + (p >> 5), j = by * 4 + ((p >> 3) & 3), k = bz * 8 + (p & 7);
+  const bool in = i < g.nx && j < g.ny && k < g.nz;
+  for (int e = ptr[t]; e < ptr[t + 1]; ++e) {
+    double s = 0.0;
+    for (int q = ek[e]; in && q < ek[e + 1]; ++q) {
+      const int key = keys[q], mu = key >> 9;
+      const int ix = ((key >> 6) & 7) - 4 + kImgMax, iy = ((key >> 3) & 7) - 4 + kImgMax,
+                iz = (key & 7) - 4 + kImgMax;
+      const long ax = ((long)mu * kImgN + ix) * g.nx + i, ay = ((long)mu * kImgN + iy) * g.ny + j,
+                 az = ((long)mu * kImgN + iz) * g.nz + k;
+      const double r2 = __dadd_rn(__dadd_rn(tb.sq[0][ax], tb.sq[1][ay]), tb.sq[2][az]);
+      if (r2 < tb.rc2[mu]) s += tb.norm[mu] * tb.ex[0][ax] * tb.ex[1][ay] * tb.ex[2][az];
+    }
+    x[(long)e * kOxP + p] = s;
+  }
+}
+
+// largest exponent field of x into *bmax
+__global__ void __launch_bounds__(256) ox_xmax_kernel(const double *x, long n, int *bmax) {
+  int m = 1;
+  for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x)
+    m = max(m, exp_field(x[e]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(bmax, m);
+}
+
+// FP64 -> fixed point in place, the points' shifts, and sum X^2 per function
+__global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int *id, int shift,
+                                                       const int *bmax, long long *x,
+                                                       signed char *rsh, double *s2) {
+  const int t = blockIdx.x, p = threadIdx.x, b = *bmax;
+  unsigned long long big = 0;
+  for (int e = ptr[t]; e < ptr[t + 1]; ++e) {
+    const double v = __longlong_as_double(x[(long)e * kOxP + p]);
+    const long long f = to_fixed(v, b);
+    x[(long)e * kOxP + p] = f;
+    big = max(big, (unsigned long long)(f < 0 ? -f : f));
+    double q = v * v;
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if ((p & 31) == 0) atomicAdd(s2 + (id[e] >> shift), q);
+  }
+  // |X| << s stays at most 2^62
+  rsh[(long)t * kOxP + p] = (signed char)(big ? max(0, __clzll((long long)big) - 2) : 0);
+}
+
+// ---- per evaluation: D and v in fixed point --------------------------------------
+// e with d < 2^2e
+__device__ __forceinline__ int ox_dexp(double d) { return (exp_field(d) - 1021) >> 1; }
+
+// D_ab 2^-(e_a + e_b) (one bit in reserve for rounding), the exponents and the
+// tiles' largest ones; diag: the offset 0 of DR (its diagonal bounds every offset)
+__global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, const double *diag, int M,
+                                                      int shift, int n_tiles, const int *ptr, const int *id,
+                                                      long long *dst, int *ee, int *ct) {
+  const long MM = (long)M * M, gtid = (long)blockIdx.x * 256 + threadIdx.x, gs = (long)gridDim.x * 256;
+  for (long q = gtid; q < n; q += gs) {
+    const long r = q % MM;
+    const int a = (int)(r / M), b = (int)(r % M);
+    dst[q] = to_fixed(D[q], 1023 + ox_dexp(diag[(long)a * (M + 1)]) + ox_dexp(diag[(long)b * (M + 1)]));
+  }
+  for (long a = gtid; a < M; a += gs) ee[a] = ox_dexp(diag[a * (M + 1)]);
+  const int lane = threadIdx.x & 31;
+  for (long t = gtid >> 5; t < n_tiles; t += gs >> 5) {
+    int m = -2000;
+    for (int e = ptr[t] + lane; e < ptr[t + 1]; e += 32)
+      m = max(m, ox_dexp(diag[(long)(id[e] >> shift) * (M + 1)]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) ct[t] = -m;
+  }
+}
+
+// X_pa 2^e_a in the tile's and the point's scale
+__device__ __forceinline__ long long ox_shift(long long x, int s) {
+  if (s >= 0) return x << s;
+  const int r = min(-s, 62);
+  return (x + (1LL << (r - 1))) >> r;
+}
+
+// partial maxima of the exponent fields of src
+__global__ void __launch_bounds__(256) ox_max_kernel(const double *src, long n, double scale, int *part) {
+  __shared__ int sm[8];
+  int m = 1;
+  for (long e = (long)blockIdx.x * 256 + threadIdx.x; e < n; e += (long)gridDim.x * 256)
+    m = max(m, exp_field(src[e] * scale));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) m = max(m, sm[q]);
+    part[blockIdx.x] = m;
+  }
+}
+__device__ __forceinline__ int ox_total_max(const int *part, int np) {
+  __shared__ int sm[8];
+  int m = (int)threadIdx.x < np ? part[threadIdx.x] : 1;
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = sm[0];
+  for (int q = 1; q < 8; ++q) m = max(m, sm[q]);
+  return m;
+}
+// v dV in tile order (0 outside the grid)
+__global__ void __launch_bounds__(256) ox_vfix_kernel(GridGeom g, int n_tiles, const double *v,
+                                                      const int *part, int np, long long *dst, int *bexp) {
+  const int b = ox_total_max(part, np);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *bexp = b;
+  for (long q = (long)blockIdx.x * 256 + threadIdx.x; q < (long)n_tiles * kOxP; q += (long)gridDim.x * 256) {
+    const int gp = ox_point(g, (int)(q / kOxP), (int)(q % kOxP));
+    dst[q] = (gp < 0 || b == kOzBad) ? 0 : to_fixed(v[gp] * g.dV, b);
+  }
+}
+
+// ---- the passes -----------------------------------------------------------------
+struct OxBars {
+  uint64_t full[kOxStages], empty[kOxStages], acc_full, acc_empty, fin;
+  uint64_t part_full[2], part_empty[2];
+  uint32_t tbase;
+  int stop;
+  __int128 part[2][4][kOxP];  // column parts of rho, two tiles in flight
+  int id[kOxBldW][kOxN], ee[kOxBldW][kOxN];  // entries of a builder warp's tile
+};
+
+// columns of pass h of a tile of n entries: 64, and the last 64, 32 or 16
+__device__ __forceinline__ int ox_cols(int n, int h) {
+  const int rem = n - h * kOxCols;
+  return rem > 32 ? 64 : rem > 16 ? 32 : 16;
+}
+
+// digit T of the eight values y (row r of a block of `rows` rows, columns h * 8 ..)
+template <int T, int N>
+__device__ __forceinline__ void ox_put(const unsigned long long (&y)[N], uint8_t *dst) {
+  uint32_t w[N / 2];
+#pragma unroll
+  for (int u = 0; u < N / 2; ++u) w[u] = pack_bf16(digit<T>(y[2 * u]), digit<T>(y[2 * u + 1]));
+  if constexpr (N == 8) *(uint4 *)dst = make_uint4(w[0], w[1], w[2], w[3]);
+  else *(uint2 *)dst = make_uint2(w[0], w[1]);
+}
+template <int N>
+__device__ __forceinline__ void ox_put_all(const unsigned long long (&y)[N], uint8_t *dst, int stride) {
+  ox_put<0, N>(y, dst);
+  ox_put<1, N>(y, dst + stride);
+  ox_put<2, N>(y, dst + 2 * stride);
+  ox_put<3, N>(y, dst + 3 * stride);
+  ox_put<4, N>(y, dst + 4 * stride);
+  ox_put<5, N>(y, dst + 5 * stride);
+  ox_put<6, N>(y, dst + 6 * stride);
+  ox_put<7, N>(y, dst + 7 * stride);
+}
+
+// floor(x y / 2^62) of two fixed-point numbers of at most 2^62
+__device__ __forceinline__ long long ox_mul62(long long x, long long y) {
+  return (long long)(((unsigned long long)__mul64hi(x, y) << 2) | ((unsigned long long)(x * y) >> 62));
+}
+
+// MMAs of one K step: digit q of A times digits 0 .. 7 - q of B, CW columns each,
+// into the orders q .. 7 (at most 256 columns per MMA)
+template <int CW, bool FRESH>
+__device__ __forceinline__ void ox_mma(uint32_t tmem, uint32_t a0, uint32_t b0) {
+  constexpr int per = 256 / CW;  // digits of B in one MMA
+#pragma unroll
+  for (int q = 0; q < kOzS; ++q) {
+    const uint64_t A = smem_desc(a0 + q * 128 * 32);
+#pragma unroll
+    for (int u = 0; u < kOzS - q; u += per) {
+      const int nd = per < kOzS - q - u ? per : kOzS - q - u;
+      if (FRESH && q == 0) mma_bf16<false>(tmem + (q + u) * CW, A, smem_desc(b0 + u * CW * 32), idesc_bf16(nd * CW));
+      else mma_bf16<true>(tmem + (q + u) * CW, A, smem_desc(b0 + u * CW * 32), idesc_bf16(nd * CW));
+    }
+  }
+}
+template <int CW>
+__device__ __forceinline__ void ox_mma_step(uint32_t tmem, uint32_t a0, bool fresh) {
+  if (fresh) ox_mma<CW, true>(tmem, a0, a0 + kOxA);
+  else ox_mma<CW, false>(tmem, a0, a0 + kOxA);
+}
+
+// RHO: density, else V; KP: entries are images, matrices per lattice offset
+template <bool RHO, bool KP>
+__global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
+  extern __shared__ __align__(1024) uint8_t dsm[];
+  __shared__ OxBars S;
+  const int tid = threadIdx.x, w = uniform(tid >> 5), lane = tid & 31;
+  if (tid == 0) {
+    for (int s = 0; s < kOxStages; ++s) {
+      mbar_init(&S.full[s], kOxBldW);
+      mbar_init(&S.empty[s], 1);
+    }
+    mbar_init(&S.acc_full, 1);
+    mbar_init(&S.acc_empty, kOxEpiW);
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&S.part_full[q], kOxEpiW - 4);  // the warps of parts 1 .. 3
+      mbar_init(&S.part_empty[q], 4);           // the warps of part 0
+    }
+    mbar_init(&S.fin, 1);
+    S.stop = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (w == 0) tmem_alloc(&S.tbase);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = uniform(S.tbase);
+  volatile int *stop = &S.stop;
+  const int M = g.g.M;
+  const long MM = (long)M * M;
+
+  if (w == kOxEpiW + kOxBldW) {
+    // --------------------------------- MMA issue ---------------------------------
+    int fill = 0, ch = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
+      const int n = uniform(g.ptr[t + 1] - g.ptr[t]), nks = RHO ? (n + 15) / 16 : kOxP / 16;
+      for (int h = 0; h * kOxCols < n && ok; ++h, ++ch) {
+        const int cw = ox_cols(n, h);
+        if (ch > 0 && !mbar_wait_warp(&S.acc_empty, (ch - 1) & 1, stop)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int ks = 0; ks < nks; ++ks, ++fill) {
+          const int s = fill % kOxStages, use = fill / kOxStages;
+          if (!mbar_wait_warp(&S.full[s], use & 1, stop)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t a0 = su32(dsm + s * kOxStage);
+          if (cw == 64) ox_mma_step<64>(tmem, a0, ks == 0);
+          else if (cw == 32) ox_mma_step<32>(tmem, a0, ks == 0);
+          else ox_mma_step<16>(tmem, a0, ks == 0);
+          mma_commit(&S.empty[s]);
+        }
+        if (ok) mma_commit(&S.acc_full);
+      }
+    }
+    if (!ok && lane == 0) atomicExch((int *)stop, 1);
+    mma_commit(&S.fin);  // every MMA issued has completed before the TMEM is released
+    mbar_wait_warp(&S.fin, 0);
+  } else if (w >= kOxEpiW) {
+    // ----------------------------- digits of each K step -----------------------------
+    // The inputs of a step are loaded while the previous one's digits are cut
+    // (one step's chain of L2 loads is about as long as its MMAs).
+    const int bt = tid - kOxEpiW * 32, bw = bt >> 5;
+    const int r = bt & 127, hh = bt >> 7;  // A: row, half of the K step
+    int fill = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
+      const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0, nks = RHO ? (n + 15) / 16 : kOxP / 16;
+      const int steps = (n + kOxCols - 1) / kOxCols * nks;
+      const int rs = RHO ? (int)g.rsh[(long)t * kOxP + r] + g.ct[t] : 0;
+      if (RHO) {  // ids and exponents of the tile's entries, a copy per warp
+        __syncwarp();
+        for (int e = lane; e < n; e += 32) {
+          const int id = __ldg(g.id + e0 + e);
+          S.id[bw][e] = id;
+          S.ee[bw][e] = __ldg(g.ee + (KP ? id >> 9 : id));
+        }
+        __syncwarp();
+      }
+      // inputs of step st: pass h = st / nks, K step ks = st % nks.  A: 8 values
+      // of row r; B: row bi of the pass, 4 consecutive K per item, cw * 4 items
+      auto load = [&](int st, long long (&xa)[8], long long (&xb)[4]) {
+        const int h = st / nks, ks = st - h * nks, cw = ox_cols(n, h);
+        const int bi = bt & (cw - 1), bq = bt / cw, be = h * kOxCols + bi;
+        const bool in = bt < cw * 4 && be < n;
+        if (RHO) {  // rows: points, K: entries
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int e = ks * 16 + hh * 8 + u;
+            xa[u] = e < n ? __ldg(g.x + (long)(e0 + e) * kOxP + r) : 0;
+          }
+          const int idb = in ? S.id[bw][be] : 0;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {  // D[b][k]
+            const int e = ks * 16 + bq * 4 + u;
+            xb[u] = 0;
+            if (in && e < n) {
+              const int ide = S.id[bw][e];
+              if (KP) {
+                const int ri = ox_ridx(g.G, idb, ide);
+                if (ri >= 0) xb[u] = __ldg(g.dfix + ri * MM + (long)(idb >> 9) * M + (ide >> 9));
+              } else {
+                xb[u] = __ldg(g.dfix + (long)idb * M + ide);
+              }
+            }
+          }
+        } else {  // rows: entries, K: points
+          const longlong2 *pa = (const longlong2 *)(g.x + (long)(e0 + r) * kOxP + ks * 16 + hh * 8);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const longlong2 z = r < n ? __ldg(pa + u) : make_longlong2(0, 0);
+            xa[2 * u] = z.x;
+            xa[2 * u + 1] = z.y;
+          }
+          const longlong2 *pb = (const longlong2 *)(g.x + (long)(e0 + be) * kOxP + ks * 16 + bq * 4);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const longlong2 z = in ? __ldg(pb + u) : make_longlong2(0, 0);
+            xb[2 * u] = z.x;
+            xb[2 * u + 1] = z.y;
+          }
+        }
+      };
+      long long xa[8], xb[4];
+      if (steps > 0) load(0, xa, xb);
+      for (int st = 0; st < steps; ++st, ++fill) {
+        const int h = st / nks, ks = st - h * nks, cw = ox_cols(n, h);
+        const int bi = bt & (cw - 1), bq = bt / cw;
+        const int s = fill % kOxStages, use = fill / kOxStages;
+        if (use > 0 && !mbar_wait(&S.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
+        uint8_t *stg = dsm + s * kOxStage;
+        unsigned long long ya[8], yb[4];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int e = ks * 16 + hh * 8 + u;
+          ya[u] = biased(RHO ? (e < n ? ox_shift(xa[u], rs + S.ee[bw][e]) : 0) : xa[u]);
+        }
+        if (RHO) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) yb[u] = biased(xb[u]);
+        } else {  // W = v X
+          const longlong2 *pv = (const longlong2 *)(g.vt + (long)t * kOxP + ks * 16 + min(bq, 3) * 4);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const longlong2 v = __ldg(pv + u);
+            yb[2 * u] = biased(ox_mul62(xb[2 * u], v.x));
+            yb[2 * u + 1] = biased(ox_mul62(xb[2 * u + 1], v.y));
+          }
+        }
+        if (st + 1 < steps) load(st + 1, xa, xb);
+        ox_put_all<8>(ya, stg + kstep_off(r, hh * 8), 128 * 32);
+        if (bt < cw * 4) ox_put_all<4>(yb, stg + kOxA + kstep_off(bi, bq * 4), cw * 32);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.full[s]);
+      }
+    }
+    if (!ok) atomicExch((int *)stop, 1);
+  } else {
+    // ------------------------------- read-out -------------------------------
+    const int quad = w & 3, part = w >> 2, row = quad * 32 + lane;
+    const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16);
+    int ch = 0, nt = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++nt) {
+      const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0;
+      const int gp = RHO ? ox_point(g.g, t, row) : 0;
+      const int rs = RHO ? (int)g.rsh[(long)t * kOxP + row] + g.ct[t] : 0;
+      const int ida = (!RHO && row < n) ? __ldg(g.id + e0 + row) : 0;
+      __int128 acc = 0;
+      for (int h = 0; h * kOxCols < n; ++h, ++ch) {
+        const int cw = ox_cols(n, h), cp = cw / 4;  // columns of this part
+        ok = __all_sync(0xffffffffu, mbar_wait(&S.acc_full, ch & 1, stop));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int c0 = 0; c0 < cp; c0 += 4) {
+          long long x4[4];  // density: X of the four columns, in flight with the accumulators
+          if (RHO) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int b = h * kOxCols + part * cp + c0 + j;
+              x4[j] = 0;
+              if (b < n)
+                x4[j] = ox_shift(__ldg(g.x + (long)(e0 + b) * kOxP + row),
+                                 rs + __ldg(g.ee + (KP ? __ldg(g.id + e0 + b) >> 9 : __ldg(g.id + e0 + b))));
+            }
+          }
+          uint32_t r[32];
+          oz_ld_issue(tbase + part * cp + c0, r, cw);
+          tmem_ld_wait(r);
+          if (c0 + 4 >= cp) {
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.acc_empty);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int b = h * kOxCols + part * cp + c0 + j;
+            long long hi = 0, lo = 0;
+            oz_add(r, j, hi, lo);
+            const __int128 T = ((__int128)hi << 32) + lo;  // |T| <= 2^75
+            if (RHO) {
+              // (a column beyond n has X = 0)
+              acc += ((__int128)(long long)(T >> 13) * x4[j]) >> 8;
+            } else if (b < n && b <= row && row < n) {
+              const long long v = g.sh >= 0 ? (long long)(T << g.sh)
+                                            : (long long)((T + ((__int128)1 << (-g.sh - 1))) >> -g.sh);
+              if (v != 0) {
+                const int idb = __ldg(g.id + e0 + b);
+                if (KP) {  // VR[n_a - n_b][mu_a][mu_b], and the transposed pair
+                  const int ri = ox_ridx(g.G, ida, idb);
+                  if (ri >= 0) {
+                    const int ma = ida >> 9, mb = idb >> 9;
+                    atomicAdd(g.V + ri * MM + (long)ma * M + mb, (unsigned long long)v);
+                    if (b != row)
+                      atomicAdd(g.V + ox_ridx(g.G, idb, ida) * MM + (long)mb * M + ma, (unsigned long long)v);
+                  }
+                } else {  // entries ascend: mu_b <= mu_a
+                  atomicAdd(g.V + (long)idb * M + ida, (unsigned long long)v);
+                  if (g.full && b != row) atomicAdd(g.V + (long)ida * M + idb, (unsigned long long)v);
+                }
+              }
+            }
+          }
+        }
+      }
+      if (!ok) break;
+      if (RHO) {
+        // the four column parts of each point, summed exactly
+        const int q = nt & 1;
+        if (part > 0) {
+          if (nt >= 2) ok = __all_sync(0xffffffffu, mbar_wait(&S.part_empty[q], ((nt >> 1) - 1) & 1, stop));
+          S.part[q][part][row] = acc;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&S.part_full[q]);
+          continue;
+        }
+        ok = __all_sync(0xffffffffu, mbar_wait(&S.part_full[q], (nt >> 1) & 1, stop));
+        acc += S.part[q][1][row] + S.part[q][2][row] + S.part[q][3][row];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.part_empty[q]);
+        if (ok && gp >= 0) {
+          const bool neg = acc < 0;
+          unsigned __int128 u = neg ? -(unsigned __int128)acc : (unsigned __int128)acc;
+          // the leading 63 bits as FP64
+          const unsigned long long top = (unsigned long long)(u >> 64);
+          const int lz = top ? __clzll((long long)top) : 64 + __clzll((long long)(unsigned long long)u);
+          const int drop = max(0, 65 - lz);
+          const double m = (double)(long long)(unsigned long long)(u >> drop);
+          const double v = oz_scale(m, drop + 2 * g.bX - 2152 - 2 * rs);
+          g.rho[gp] = neg ? -v : v;
+        }
+      }
+    }
+    if (!ok) atomicExch((int *)stop, 1);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (w == 0) tmem_dealloc(tmem);
+  if (tid == 0 && S.stop) atomicExch(g.flags + FLAG_ERR, ETDM_ERR_TIMEOUT);
+}
+
+// H += the fixed-point sums (upper triangle), unit 2^(bV + hexp - 1084)
+__global__ void __launch_bounds__(256) ox_vadd_kernel(const unsigned long long *V, int M, int hexp,
+                                                      const int *bexp, double *H) {
+  const int b = *bexp;
+  const long MM = (long)M * M;
+  for (long e = (long)blockIdx.x * 256 + threadIdx.x; e < MM; e += (long)gridDim.x * 256) {
+    if (e / M > e % M) continue;
+    H[e] += b == kOzBad ? nan("") : oz_scale((double)(long long)V[e], b + hexp - 1084);
+  }
+}
+// the sums as FP64, in place
+__global__ void __launch_bounds__(256) ox_vcvt_kernel(double *V, long n, int hexp, const int *bexp) {
+  const int b = *bexp;
+  for (long e = (long)blockIdx.x * 256 + threadIdx.x; e < n; e += (long)gridDim.x * 256) {
+    const long long q = __double_as_longlong(V[e]);
+    V[e] = b == kOzBad ? nan("") : oz_scale((double)q, b + hexp - 1084);
+  }
+}
+
+// ---- host side -------------------------------------------------------------------
+namespace {
+
+OxArgs ox_args(etdm_handle *h) {
+  const OxGrid &o = h->ox;
+  OxArgs a{};
+  a.g = o.geom;
+  a.G = h->kg;
+  a.n_tiles = o.n_tiles;
+  a.bX = o.bX;
+  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.rsh = o.rsh;
+  a.dfix = o.dfix; a.ee = o.ee; a.ct = o.ct; a.bexp = o.bexp; a.vt = o.vt;
+  a.flags = h->d_flags;
+  return a;
+}
+
+template <bool RHO, bool KP>
+cudaError_t ox_launch(const OxArgs &a, int sms, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(ox_pass_kernel<RHO, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kOxStages * kOxStage);
+  if (e != cudaSuccess) return e;
+  ox_pass_kernel<RHO, KP><<<std::min(a.n_tiles, sms), kOxThreads, kOxStages * kOxStage, s>>>(a);
+  return cudaGetLastError();
+}
+
+int ox_parts(long n) { return (int)std::max<long>(1, std::min<long>(kOxParts, (n + 2047) / 2048)); }
+
+}  // namespace
+
+// Tables of the passes from the 4 x 4 x 8 tiles' image lists (ptr, keys on the
+// host and on the device).  `images`: one entry per image, else per function.
+// Leaves h->ox.n_tiles = 0 (the passes of grid.cu run) when a tile has more
+// than 128 entries or the memory for X is not there.
+void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vector<int> &kptr,
+              const std::vector<int> &keys, const int *d_keys, bool images, cudaStream_t s) {
+  OxGrid &o = h->ox;
+  std::vector<int> ptr(n_tiles + 1, 0), id, ek;
+  for (int t = 0; t < n_tiles; ++t) {
+    for (int e = kptr[t]; e < kptr[t + 1]; ++e)
+      if (images || e == kptr[t] || (keys[e] >> 9) != (keys[e - 1] >> 9)) {
+        id.push_back(images ? keys[e] : keys[e] >> 9);
+        ek.push_back(e);
+      }
+    ptr[t + 1] = (int)id.size();
+    if (ptr[t + 1] - ptr[t] > kOxN) return;
+  }
+  const long ne = (long)id.size();
+  if (ne == 0) return;
+  ek.push_back((int)keys.size());
+  const long mats = images ? h->kg.nR : 1, MM = (long)h->M * h->M;
+  const size_t bytes = (size_t)ne * kOxP * 8 + (size_t)n_tiles * kOxP * 9 + (size_t)mats * MM * 8 +
+                       (h->kpath ? 0 : (size_t)MM * 8) + 4096;
+  unsigned char *p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  h->allocs.push_back(p);
+  auto take = [&p](size_t n) {
+    unsigned char *q = p;
+    p += (n + 255) & ~(size_t)255;
+    return q;
+  };
+  o.x = (long long *)take((size_t)ne * kOxP * 8);
+  o.vt = (long long *)take((size_t)n_tiles * kOxP * 8);
+  o.dfix = (long long *)take((size_t)mats * MM * 8);
+  if (!h->kpath) o.V = (unsigned long long *)take((size_t)MM * 8);
+  o.rsh = (signed char *)take((size_t)n_tiles * kOxP);
+  o.ptr = dupload(h, ptr.data(), ptr.size());
+  o.id = dupload(h, id.data(), id.size());
+  o.part = dalloc<int>(h, kOxParts);
+  o.bexp = dalloc<int>(h, 1);
+  o.ee = dalloc<int>(h, h->M);
+  o.ct = dalloc<int>(h, n_tiles);
+  int *d_ek = dupload(h, ek.data(), ek.size());
+  int *d_b = dalloc<int>(h, 1);
+  double *d_s2 = dalloc<double>(h, h->M);
+  Tables tb;
+  for (int a = 0; a < 3; ++a) {
+    tb.sq[a] = h->d_sq + h->tab_off[a];
+    tb.ex[a] = h->d_ex + h->tab_off[a];
+  }
+  tb.norm = h->d_norm;
+  tb.rc2 = h->d_rc2;
+  ox_basis_kernel<<<n_tiles, kOxP, 0, s>>>(geom, tb, o.ptr, d_ek, d_keys, (double *)o.x);
+  CUDA_TRY(cudaGetLastError());
+  ox_xmax_kernel<<<1024, 256, 0, s>>>((const double *)o.x, ne * kOxP, d_b);
+  CUDA_TRY(cudaGetLastError());
+  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, images ? 9 : 0, d_b, o.x, o.rsh, d_s2);
+  CUDA_TRY(cudaGetLastError());
+  std::vector<double> s2(h->M);
+  CUDA_TRY(cudaMemcpy(&o.bX, d_b, sizeof(int), cudaMemcpyDeviceToHost));
+  CUDA_TRY(cudaMemcpy(s2.data(), d_s2, h->M * 8, cudaMemcpyDeviceToHost));
+  dfree(h, d_ek);
+  dfree(h, d_b);
+  dfree(h, d_s2);
+  double mx = 0.0;
+  for (double v : s2) mx = std::max(mx, v);
+  if (o.bX == kOzBad || !std::isfinite(mx)) return;
+  o.hexp = ilogb(std::max(mx, 1e-300)) + 1;
+  o.geom = geom;
+  o.images = images;
+  o.n_tiles = n_tiles;
+}
+
+// rho on the grid from D [M][M] (Gamma point) or DR [offset][M][M]
+cudaError_t launch_ox_rho(etdm_handle *h, const double *D, double *rho, cudaStream_t s) {
+  const OxGrid &o = h->ox;
+  const long n = (o.images ? (long)h->kg.nR : 1L) * h->M * h->M;
+  const long work = std::max(n, (long)o.n_tiles * 32);
+  ox_dfix_kernel<<<(int)std::min<long>(8 * h->num_sms, (work + 255) / 256), 256, 0, s>>>(
+      D, n, D + (o.images ? (h->kg.nR - 1) / 2 : 0) * (long)h->M * h->M, h->M, o.images ? 9 : 0, o.n_tiles,
+      o.ptr, o.id, o.dfix, o.ee, o.ct);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  OxArgs a = ox_args(h);
+  a.rho = rho;
+  return o.images ? ox_launch<true, true>(a, h->num_sms, s) : ox_launch<true, false>(a, h->num_sms, s);
+}
+
+namespace {
+// V of the potential v into the zeroed sums V
+cudaError_t ox_vmat(etdm_handle *h, const double *v, unsigned long long *V, bool full, cudaStream_t s) {
+  const OxGrid &o = h->ox;
+  const int np = ox_parts(h->G);
+  ox_max_kernel<<<np, 256, 0, s>>>(v, h->G, o.geom.dV, o.part);
+  ox_vfix_kernel<<<(int)std::min<long>(4 * h->num_sms, ((long)o.n_tiles * kOxP + 255) / 256), 256, 0, s>>>(
+      o.geom, o.n_tiles, v, o.part, np, o.vt, o.bexp);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  OxArgs a = ox_args(h);
+  a.V = V;
+  a.full = full;
+  a.sh = 2 * o.bX - o.hexp - 2050;
+  return o.images ? ox_launch<false, true>(a, h->num_sms, s) : ox_launch<false, false>(a, h->num_sms, s);
+}
+}  // namespace
+
+// H (upper triangle) += V
+cudaError_t launch_ox_vmat(etdm_handle *h, const double *v, double *H, cudaStream_t s) {
+  const OxGrid &o = h->ox;
+  const long MM = (long)h->M * h->M;
+  cudaError_t e = cudaMemsetAsync(o.V, 0, MM * 8, s);
+  if (e != cudaSuccess) return e;
+  if ((e = ox_vmat(h, v, o.V, false, s)) != cudaSuccess) return e;
+  ox_vadd_kernel<<<(int)std::min<long>(4 * h->num_sms, (MM + 255) / 256), 256, 0, s>>>(o.V, h->M, o.hexp, o.bexp, H);
+  return cudaGetLastError();
+}
+
+// VR [offset][M][M] = V (overwritten)
+cudaError_t launch_ox_vmat_k(etdm_handle *h, const double *v, double *VR, cudaStream_t s) {
+  const OxGrid &o = h->ox;
+  const long n = (long)h->kg.nR * h->M * h->M;
+  cudaError_t e = cudaMemsetAsync(VR, 0, n * 8, s);
+  if (e != cudaSuccess) return e;
+  if ((e = ox_vmat(h, v, (unsigned long long *)VR, true, s)) != cudaSuccess) return e;
+  ox_vcvt_kernel<<<(int)std::min<long>(8 * h->num_sms, (n + 255) / 256), 256, 0, s>>>(VR, n, o.hexp, o.bexp);
+  return cudaGetLastError();
+}
+
+}  // namespace etdm
