@@ -302,7 +302,7 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
                     E, h->d_flags, s, h->sic ? h->d_sicpart : nullptr,
                     h->sic ? h->N * pot_blocks(h) : 0));
   // exp: iA, the eigensolver and the phases (eig); O f, DR, density, 5 potential passes, 2 energy sums
-  h->launches += (ss ? 0 : 2 + heev_launches(M, &h->oz)) + 9 + rho64_launches(h);
+  h->launches += (ss ? 0 : 2 + heev_launches(M, nk, &h->oz)) + 9 + rho64_launches(h);
   if (!g) {
     tk.done();
     return;

@@ -53,7 +53,7 @@ size_t heev_work_bytes(int n, int batch);
 // reflectors on the tensor cores (their workspace; null: reflector by reflector)
 cudaError_t launch_heev(double2 *A, double *w, double2 *V, int n, int batch, void *work,
                         int *flags, cudaStream_t s, int method = 0, const OzWork *oz = nullptr);
-int heev_launches(int n, const OzWork *oz);  // kernels of one call with method 1
+int heev_launches(int n, int batch, const OzWork *oz);  // kernels of one call with method 1
 
 
 }  // namespace etdm

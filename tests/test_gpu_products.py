@@ -2,7 +2,9 @@
 wrong, through E and the gradient against the k-point oracle: FP64 tiles with
 a remainder and one k-point (20), the largest on the FP64 kernel (64), tensor
 cores with a K tail and a partial column tile (80), a second block of 128 rows
-(144); with exp(A) by both routes."""
+(144); the eigensolver's panels of 16 columns from the first size that takes
+them, whole (128) and with a remainder of 7 (135), for eight matrices and for
+one, whose blocks hold a few rows each; with exp(A) by both routes."""
 import numpy as np
 import pytest
 
@@ -16,6 +18,8 @@ SYSTEMS = {
     64: dict(cells=(2, 2, 2), n_exp=8, grid=(16, 15, 14), kmesh=2),
     80: dict(cells=(2, 5, 2), n_exp=4, grid=(14, 24, 15), kmesh=2),
     144: dict(cells=(3, 3, 4), n_exp=4, grid=(20, 18, 24), kmesh=2),
+    128: dict(cells=(4, 2, 4), n_exp=4, grid=(24, 15, 24), kmesh=1),
+    135: dict(cells=(3, 3, 5), n_exp=3, grid=(20, 18, 28), kmesh=2),
 }
 
 
