@@ -1339,6 +1339,12 @@ __global__ void __launch_bounds__(NT) dense_reverse_batch_kernel(const DenseArgs
   }
 }
 
+}  // namespace etdm
+
+#include "dense_small.cuh"
+
+namespace etdm {
+
 // The float-pair chains with their large products on the tensor cores: one
 // block per SM (the stage ring's dynamic shared memory leaves room for no
 // second block), 512 tensor-memory columns held for the kernel's lifetime.
@@ -1820,10 +1826,28 @@ DenseArgs dense_args(etdm_handle *h, const double *a) {
   return d;
 }
 
+// One block with all matrices in shared memory: where the general chains would
+// run on one block too and the matrices fit
+static bool takes_small(const etdm_handle *h) {
+  return h->coop_blocks == 1 && !(dense_pairs(h) && h->dense_tc) && small_fits(h->M, h->N, h->V);
+}
+template <class K, class... T>
+static cudaError_t launch_small(K kernel, int sm, cudaStream_t s, T... args) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallBytes);
+  if (e != cudaSuccess) return e;
+  kernel<<<1, NT, sm, s>>>(args...);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_dense_forward(etdm_handle *h, const double *a, cudaStream_t s) {
   DenseArgs d = dense_args(h, a);
   void *args[] = {&d};
   h->pairs_last = dense_pairs(h);
+  if (takes_small(h)) {
+    const int sm = SmallFwd(d.M, d.N, d.V).total * 8;
+    return dense_pairs(h) ? launch_small(dense_forward_small_kernel<float2>, sm, s, d)
+                          : launch_small(dense_forward_small_kernel<double>, sm, s, d);
+  }
   if (dense_pairs(h) && h->dense_tc)
     return cudaLaunchCooperativeKernel((const void *)dense_forward_tc_kernel, dim3(h->coop_blocks),
                                        dim3(NT), args, kGDyn, s);
@@ -1838,6 +1862,11 @@ cudaError_t launch_dense_reverse(etdm_handle *h, const double *a, double *g, dou
   d.g = g; d.E = E;
   d.resid = (h->want_resid && g) ? h->d_dot + 3 : nullptr;  // Eq. 45 with the energy
   int want = g != nullptr;
+  if (takes_small(h)) {
+    const int sm = SmallRev(d.M, d.N, d.V).total * 8;
+    return dense_pairs(h) ? launch_small(dense_reverse_small_kernel<float2>, sm, s, d, want)
+                          : launch_small(dense_reverse_small_kernel<double>, sm, s, d, want);
+  }
   void *args[] = {&d, &want};
   if (dense_pairs(h) && h->dense_tc)
     return cudaLaunchCooperativeKernel((const void *)dense_reverse_tc_kernel, dim3(h->coop_blocks),
