@@ -291,12 +291,18 @@ GridGeom make_geom(etdm_handle *h, int tx, int ty, int tz, int *n_tiles) {
 // Truncation lists of one tile geometry: count per (tile, mu), exclusive scan,
 // fill in (tile, mu, image) order (sorted keys within a tile).
 void build_lists(etdm_handle *h, const GridGeom &g, int n_tiles, int **d_ptr, int **d_keys,
-                 long *n_entries, int *max_list, int limit, cudaStream_t s) {
+                 long *n_entries, int *max_list, int limit, cudaStream_t s,
+                 std::vector<int> *host_ptr = nullptr) {
   const int M = h->M;
   const long ncnt = (long)n_tiles * M;
-  int *d_count = dalloc<int>(h, ncnt);
-  long long *d_off = dalloc<long long>(h, ncnt);
-  long long *d_tmp = dalloc<long long>(h, ncnt / 1024 + 4);
+  if (ncnt > h->list_cap) {  // (the first geometry has the most tiles; the next ones reuse its scratch)
+    h->d_lcount = dalloc<int>(h, ncnt);
+    h->d_loff = dalloc<long long>(h, ncnt);
+    h->d_ltmp = dalloc<long long>(h, ncnt / 1024 + 4);
+    h->list_cap = ncnt;
+  }
+  int *const d_count = h->d_lcount;
+  long long *const d_off = h->d_loff, *const d_tmp = h->d_ltmp;
   CUDA_TRY(launch_list_count(h, g, n_tiles, d_count, s));
   CUDA_TRY(launch_scan(d_count, d_off, ncnt, d_tmp, s));
   long nb = (ncnt + 1023) / 1024;
@@ -314,6 +320,7 @@ void build_lists(etdm_handle *h, const GridGeom &g, int n_tiles, int **d_ptr, in
   CUDA_TRY(cudaMemcpy(ptr.data(), *d_ptr, (n_tiles + 1) * sizeof(int), cudaMemcpyDeviceToHost));
   *max_list = 0;
   for (int t = 0; t < n_tiles; ++t) *max_list = std::max(*max_list, ptr[t + 1] - ptr[t]);
+  if (host_ptr) host_ptr->swap(ptr);
   if (*max_list > limit)
     throw Fail{ETDM_ERR_INVALID_ARG,
                "a " + std::to_string(g.tx) + "x" + std::to_string(g.ty) + "x" +
@@ -381,9 +388,9 @@ void etdm::setup_ox(etdm_handle *h, bool images, cudaStream_t s) {
   int T = 0, max_list = 0, *d_ptr = nullptr, *d_keys = nullptr;
   long n = 0;
   const GridGeom geom = make_geom(h, 4, 4, 8, &T);
-  build_lists(h, geom, T, &d_ptr, &d_keys, &n, &max_list, INT32_MAX, s);
-  std::vector<int> ptr(T + 1), keys(n);
-  CUDA_TRY(cudaMemcpy(ptr.data(), d_ptr, (T + 1) * sizeof(int), cudaMemcpyDeviceToHost));
+  std::vector<int> ptr;
+  build_lists(h, geom, T, &d_ptr, &d_keys, &n, &max_list, INT32_MAX, s, &ptr);
+  std::vector<int> keys(n);
   if (n > 0) CUDA_TRY(cudaMemcpy(keys.data(), d_keys, n * sizeof(int), cudaMemcpyDeviceToHost));
   ox_setup(h, geom, T, ptr, keys, d_keys, images, s);
   dfree(h, d_ptr);

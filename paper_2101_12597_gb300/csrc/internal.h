@@ -298,7 +298,7 @@ struct OxGrid {
   bool images = false;          // entries are images (k-points), else functions
   int bX = 0, hexp = 0;         // exponents of X and of V's fixed point
   int *ptr = nullptr, *id = nullptr;
-  long long *x = nullptr, *vt = nullptr, *dfix = nullptr;
+  long long *x = nullptr, *xt = nullptr, *vt = nullptr, *dfix = nullptr;
   unsigned long long *V = nullptr;
   signed char *rsh = nullptr;
   int *part = nullptr, *bexp = nullptr, *ee = nullptr, *ct = nullptr;
@@ -427,6 +427,11 @@ struct etdm_handle {
   double *d_bar2[4] = {nullptr};
   double *d_Wr = nullptr;
   double *d_Abar = nullptr;
+  // scratch of the truncation lists' construction, list_cap counts
+  int *d_lcount = nullptr;
+  long long *d_loff = nullptr, *d_ltmp = nullptr;
+  long list_cap = 0;
+
   // grid
   double *d_vext = nullptr, *d_rho = nullptr, *d_vtot = nullptr;
   double2 *d_fft = nullptr;

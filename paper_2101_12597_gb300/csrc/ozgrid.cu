@@ -29,13 +29,24 @@
 //      bound of |V_ab|, max |v dV| times the largest sum of X^2 of a function
 //      (sums wrap harmlessly in between).
 //
-// One persistent block per SM: warps 0-15 read the accumulators (lane quarter
-// w % 4, column quarter w / 4), warps 16-23 cut the digits of a K step of 16
-// into a four-stage ring, warp 24 issues the MMAs.  The columns of a tile go in
-// passes of 64 (eight orders of 64 columns fill tensor memory), the last one
-// 64, 32 or 16 wide.  A tile's K is at most 128, one exact chunk.
+// One persistent block per SM: warps 0-7 read the accumulators (lane quarter
+// w % 4, column half w / 4), two sets of eight warps cut the digits of the K
+// steps of 16 in turn into a four-stage ring, warp 24 issues the MMAs.  The
+// columns of a tile go in passes of 64 (eight orders of 64 columns fill tensor
+// memory), the last one 64, 32 or 16 wide.  A tile's K is at most 128, one exact
+// chunk.
+//
+// What bounds it: a K step's MMAs take 1152 tensor cycles, its digits some 3500
+// instructions and a column's read-out 50 per warp, and the three do not overlap
+// fully (the accumulators fill tensor memory).  The inputs of a step are loaded
+// a step of the set ahead, by lanes along consecutive elements: X is kept twice,
+// [entry][point] for the density and [pair of points][entry] for V, and D is
+// read by its columns.  With one set of builders and V's rows 1 KB apart, D's
+// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.08 and
+// 1.07 ms (11.2 and 9.4 ms on the FP64 pipe).
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
@@ -53,8 +64,10 @@ constexpr int kOxCols = 64;                     // columns of a pass, at most
 constexpr int kOxA = kOzS * 128 * 32, kOxB = kOzS * kOxCols * 32;
 constexpr int kOxStage = kOxA + kOxB;           // 48 KB
 constexpr int kOxStages = 4;
-constexpr int kOxEpiW = 16, kOxBldW = 8;
-constexpr int kOxThreads = (kOxEpiW + kOxBldW + 1) * 32;
+constexpr int kOxEpiW = 8, kOxBldW = 8, kOxSets = 2;  // warps: read-out, of a builder set
+constexpr int kOxEpiP = kOxEpiW / 4;            // column parts of the read-out
+constexpr int kOxMmaW = kOxEpiW + kOxSets * kOxBldW;
+constexpr int kOxThreads = (kOxMmaW + 1) * 32;
 constexpr int kOxParts = 256;                   // partial maxima of a fixed-point conversion
 
 struct OxArgs {
@@ -62,7 +75,8 @@ struct OxArgs {
   KGeom G;                  // lattice offsets (k-points)
   int n_tiles, bX;          // |X| < 2^(bX - 1022)
   const int *ptr, *id;      // entries of a tile; mu, or the image key (k-points)
-  const long long *x;       // [entry][128]
+  const long long *x;       // [entry][128] (density)
+  const long long *xt;      // V: per tile [64 pairs of points][entry][2]
   const signed char *rsh;   // [tile][128] left shift that fills a point's largest |X|
   const long long *dfix;    // density: scaled D, or DR per offset
   const int *ee, *ct;       // density: exponents e_a of the functions; -max e_a of a tile
@@ -125,13 +139,15 @@ __global__ void __launch_bounds__(256) ox_xmax_kernel(const double *x, long n, i
 // FP64 -> fixed point in place, the points' shifts, and sum X^2 per function
 __global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int *id, int shift,
                                                        const int *bmax, long long *x,
-                                                       signed char *rsh, double *s2) {
-  const int t = blockIdx.x, p = threadIdx.x, b = *bmax;
+                                                       long long *xt, signed char *rsh, double *s2) {
+  const int t = blockIdx.x, p = threadIdx.x, b = *bmax, n = ptr[t + 1] - ptr[t];
+  long long *const xp = xt + (long)ptr[t] * kOxP + (long)(p >> 1) * n * 2 + (p & 1);
   unsigned long long big = 0;
   for (int e = ptr[t]; e < ptr[t + 1]; ++e) {
     const double v = __longlong_as_double(x[(long)e * kOxP + p]);
     const long long f = to_fixed(v, b);
     x[(long)e * kOxP + p] = f;
+    xp[2 * (e - ptr[t])] = f;
     big = max(big, (unsigned long long)(f < 0 ? -f : f));
     double q = v * v;
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
@@ -215,8 +231,8 @@ struct OxBars {
   uint64_t part_full[2], part_empty[2];
   uint32_t tbase;
   int stop;
-  __int128 part[2][4][kOxP];  // column parts of rho, two tiles in flight
-  int id[kOxBldW][kOxN], ee[kOxBldW][kOxN];  // entries of a builder warp's tile
+  __int128 part[2][kOxEpiP - 1][kOxP];  // column parts of rho, two tiles in flight
+  int id[kOxSets * kOxBldW][kOxN], ee[kOxSets * kOxBldW][kOxN];  // entries of a builder warp's tile
 };
 
 // columns of pass h of a tile of n entries: 64, and the last 64, 32 or 16
@@ -287,7 +303,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
     mbar_init(&S.acc_full, 1);
     mbar_init(&S.acc_empty, kOxEpiW);
     for (int q = 0; q < 2; ++q) {
-      mbar_init(&S.part_full[q], kOxEpiW - 4);  // the warps of parts 1 .. 3
+      mbar_init(&S.part_full[q], kOxEpiW - 4);  // the warps of the parts from 1 up
       mbar_init(&S.part_empty[q], 4);           // the warps of part 0
     }
     mbar_init(&S.fin, 1);
@@ -303,7 +319,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
   const int M = g.g.M;
   const long MM = (long)M * M;
 
-  if (w == kOxEpiW + kOxBldW) {
+  if (w == kOxMmaW) {
     // --------------------------------- MMA issue ---------------------------------
     int fill = 0, ch = 0;
     bool ok = true;
@@ -333,9 +349,10 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
     // ----------------------------- digits of each K step -----------------------------
     // The inputs of a step are loaded while the previous one's digits are cut
     // (one step's chain of L2 loads is about as long as its MMAs).
-    const int bt = tid - kOxEpiW * 32, bw = bt >> 5;
+    // The sets take the steps in turn.
+    const int bw = w - kOxEpiW, set = bw / kOxBldW, bt = tid - (kOxEpiW + set * kOxBldW) * 32;
     const int r = bt & 127, hh = bt >> 7;  // A: row, half of the K step
-    int fill = 0;
+    int first = 0;                         // steps of the tiles before
     bool ok = true;
     for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0, nks = RHO ? (n + 15) / 16 : kOxP / 16;
@@ -352,7 +369,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       }
       // inputs of step st: pass h = st / nks, K step ks = st % nks.  A: 8 values
       // of row r; B: row bi of the pass, 4 consecutive K per item, cw * 4 items
-      auto load = [&](int st, long long (&xa)[8], long long (&xb)[4]) {
+      auto load = [&](int st, long long (&xa)[8], long long (&xb)[4], longlong2 (&xv)[2]) {
         const int h = st / nks, ks = st - h * nks, cw = ox_cols(n, h);
         const int bi = bt & (cw - 1), bq = bt / cw, be = h * kOxCols + bi;
         const bool in = bt < cw * 4 && be < n;
@@ -364,39 +381,43 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           }
           const int idb = in ? S.id[bw][be] : 0;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {  // D[b][k]
+          for (int u = 0; u < 4; ++u) {  // D[k][b] = D[b][k]: the lanes along b read consecutive elements
             const int e = ks * 16 + bq * 4 + u;
             xb[u] = 0;
             if (in && e < n) {
               const int ide = S.id[bw][e];
               if (KP) {
-                const int ri = ox_ridx(g.G, idb, ide);
-                if (ri >= 0) xb[u] = __ldg(g.dfix + ri * MM + (long)(idb >> 9) * M + (ide >> 9));
+                const int ri = ox_ridx(g.G, ide, idb);
+                if (ri >= 0) xb[u] = __ldg(g.dfix + ri * MM + (long)(ide >> 9) * M + (idb >> 9));
               } else {
-                xb[u] = __ldg(g.dfix + (long)idb * M + ide);
+                xb[u] = __ldg(g.dfix + (long)ide * M + idb);
               }
             }
           }
         } else {  // rows: entries, K: points
-          const longlong2 *pa = (const longlong2 *)(g.x + (long)(e0 + r) * kOxP + ks * 16 + hh * 8);
+          const longlong2 *px = (const longlong2 *)(g.xt + (long)e0 * kOxP) + (long)ks * 8 * n;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const longlong2 z = r < n ? __ldg(pa + u) : make_longlong2(0, 0);
+            const longlong2 z = r < n ? __ldg(px + (hh * 4 + u) * n + r) : make_longlong2(0, 0);
             xa[2 * u] = z.x;
             xa[2 * u + 1] = z.y;
           }
-          const longlong2 *pb = (const longlong2 *)(g.x + (long)(e0 + be) * kOxP + ks * 16 + bq * 4);
+          const longlong2 *pv = (const longlong2 *)(g.vt + (long)t * kOxP + ks * 16 + min(bq, 3) * 4);
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            const longlong2 z = in ? __ldg(pb + u) : make_longlong2(0, 0);
+            const longlong2 z = in ? __ldg(px + (bq * 2 + u) * n + be) : make_longlong2(0, 0);
             xb[2 * u] = z.x;
             xb[2 * u + 1] = z.y;
+            xv[u] = __ldg(pv + u);
           }
         }
       };
       long long xa[8], xb[4];
-      if (steps > 0) load(0, xa, xb);
-      for (int st = 0; st < steps; ++st, ++fill) {
+      longlong2 xv[2];
+      const int st0 = (set + kOxSets - first % kOxSets) % kOxSets;
+      if (st0 < steps) load(st0, xa, xb, xv);
+      for (int st = st0; st < steps; st += kOxSets) {
+        const int fill = first + st;
         const int h = st / nks, ks = st - h * nks, cw = ox_cols(n, h);
         const int bi = bt & (cw - 1), bq = bt / cw;
         const int s = fill % kOxStages, use = fill / kOxStages;
@@ -412,21 +433,20 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) yb[u] = biased(xb[u]);
         } else {  // W = v X
-          const longlong2 *pv = (const longlong2 *)(g.vt + (long)t * kOxP + ks * 16 + min(bq, 3) * 4);
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            const longlong2 v = __ldg(pv + u);
-            yb[2 * u] = biased(ox_mul62(xb[2 * u], v.x));
-            yb[2 * u + 1] = biased(ox_mul62(xb[2 * u + 1], v.y));
+            yb[2 * u] = biased(ox_mul62(xb[2 * u], xv[u].x));
+            yb[2 * u + 1] = biased(ox_mul62(xb[2 * u + 1], xv[u].y));
           }
         }
-        if (st + 1 < steps) load(st + 1, xa, xb);
+        if (st + kOxSets < steps) load(st + kOxSets, xa, xb, xv);
         ox_put_all<8>(ya, stg + kstep_off(r, hh * 8), 128 * 32);
         if (bt < cw * 4) ox_put_all<4>(yb, stg + kOxA + kstep_off(bi, bq * 4), cw * 32);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.full[s]);
       }
+      first += steps;
     }
     if (!ok) atomicExch((int *)stop, 1);
   } else {
@@ -439,24 +459,40 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0;
       const int gp = RHO ? ox_point(g.g, t, row) : 0;
       const int rs = RHO ? (int)g.rsh[(long)t * kOxP + row] + g.ct[t] : 0;
-      const int ida = (!RHO && row < n) ? __ldg(g.id + e0 + row) : 0;
+      // ids (V) or exponents (density) of the tile's entries, entry lane + 32 q
+      int ent[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int e = lane + 32 * q;
+        ent[q] = e < n ? __ldg(g.id + e0 + e) : 0;
+        if (RHO && e < n) ent[q] = __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q]));
+      }
+      auto entry = [&](int b) {  // (b: the same in every lane)
+        const int lo = b & 32 ? ent[1] : ent[0], hi = b & 32 ? ent[3] : ent[2];
+        return __shfl_sync(0xffffffffu, b & 64 ? hi : lo, b & 31);
+      };
+      const int ida = RHO ? 0 : ent[quad];  // entry `row`
+      // density: X of the next four columns, loaded a group ahead
+      long long xn[4];
+      auto ahead = [&](int b0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xn[j] = b0 + j < n ? __ldg(g.x + (long)(e0 + b0 + j) * kOxP + row) : 0;
+      };
+      if (RHO) ahead(part * (ox_cols(n, 0) / kOxEpiP));
       __int128 acc = 0;
       for (int h = 0; h * kOxCols < n; ++h, ++ch) {
-        const int cw = ox_cols(n, h), cp = cw / 4;  // columns of this part
+        const int cw = ox_cols(n, h), cp = cw / kOxEpiP;  // columns of this part
         ok = __all_sync(0xffffffffu, mbar_wait(&S.acc_full, ch & 1, stop));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         for (int c0 = 0; c0 < cp; c0 += 4) {
-          long long x4[4];  // density: X of the four columns, in flight with the accumulators
+          const int b0 = h * kOxCols + part * cp + c0;
+          long long x4[4];
           if (RHO) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int b = h * kOxCols + part * cp + c0 + j;
-              x4[j] = 0;
-              if (b < n)
-                x4[j] = ox_shift(__ldg(g.x + (long)(e0 + b) * kOxP + row),
-                                 rs + __ldg(g.ee + (KP ? __ldg(g.id + e0 + b) >> 9 : __ldg(g.id + e0 + b))));
-            }
+            for (int j = 0; j < 4; ++j) x4[j] = ox_shift(xn[j], rs + entry(b0 + j));
+            const int b1 = c0 + 4 < cp ? b0 + 4 : (h + 1) * kOxCols + part * (ox_cols(n, h + 1) / kOxEpiP);
+            if (c0 + 4 < cp || (h + 1) * kOxCols < n) ahead(b1);
           }
           uint32_t r[32];
           oz_ld_issue(tbase + part * cp + c0, r, cw);
@@ -468,7 +504,8 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const int b = h * kOxCols + part * cp + c0 + j;
+            const int b = b0 + j;
+            const int idb = RHO ? 0 : entry(b);
             long long hi = 0, lo = 0;
             oz_add(r, j, hi, lo);
             const __int128 T = ((__int128)hi << 32) + lo;  // |T| <= 2^75
@@ -479,7 +516,6 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
               const long long v = g.sh >= 0 ? (long long)(T << g.sh)
                                             : (long long)((T + ((__int128)1 << (-g.sh - 1))) >> -g.sh);
               if (v != 0) {
-                const int idb = __ldg(g.id + e0 + b);
                 if (KP) {  // VR[n_a - n_b][mu_a][mu_b], and the transposed pair
                   const int ri = ox_ridx(g.G, ida, idb);
                   if (ri >= 0) {
@@ -499,17 +535,18 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       }
       if (!ok) break;
       if (RHO) {
-        // the four column parts of each point, summed exactly
+        // the column parts of each point, summed exactly
         const int q = nt & 1;
         if (part > 0) {
           if (nt >= 2) ok = __all_sync(0xffffffffu, mbar_wait(&S.part_empty[q], ((nt >> 1) - 1) & 1, stop));
-          S.part[q][part][row] = acc;
+          S.part[q][part - 1][row] = acc;
           __syncwarp();
           if (lane == 0) mbar_arrive(&S.part_full[q]);
           continue;
         }
         ok = __all_sync(0xffffffffu, mbar_wait(&S.part_full[q], (nt >> 1) & 1, stop));
-        acc += S.part[q][1][row] + S.part[q][2][row] + S.part[q][3][row];
+#pragma unroll
+        for (int c = 0; c < kOxEpiP - 1; ++c) acc += S.part[q][c][row];
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.part_empty[q]);
         if (ok && gp >= 0) {
@@ -562,7 +599,7 @@ OxArgs ox_args(etdm_handle *h) {
   a.G = h->kg;
   a.n_tiles = o.n_tiles;
   a.bX = o.bX;
-  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.rsh = o.rsh;
+  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.xt = o.xt; a.rsh = o.rsh;
   a.dfix = o.dfix; a.ee = o.ee; a.ct = o.ct; a.bexp = o.bexp; a.vt = o.vt;
   a.flags = h->d_flags;
   return a;
@@ -584,7 +621,8 @@ int ox_parts(long n) { return (int)std::max<long>(1, std::min<long>(kOxParts, (n
 // Tables of the passes from the 4 x 4 x 8 tiles' image lists (ptr, keys on the
 // host and on the device).  `images`: one entry per image, else per function.
 // Leaves h->ox.n_tiles = 0 (the passes of grid.cu run) when a tile has more
-// than 128 entries or the memory for X is not there.
+// than 128 entries or the tables (2 KB per entry) would take more than half of
+// the free memory.
 void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vector<int> &kptr,
               const std::vector<int> &keys, const int *d_keys, bool images, cudaStream_t s) {
   OxGrid &o = h->ox;
@@ -602,9 +640,15 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   if (ne == 0) return;
   ek.push_back((int)keys.size());
   const long mats = images ? h->kg.nR : 1, MM = (long)h->M * h->M;
-  const size_t bytes = (size_t)ne * kOxP * 8 + (size_t)n_tiles * kOxP * 9 + (size_t)mats * MM * 8 +
-                       (h->kpath ? 0 : (size_t)MM * 8) + 4096;
-  unsigned char *p = nullptr;
+  const size_t nptr = ptr.size(), nV = h->kpath ? 0 : (size_t)MM, nint = nptr + id.size() + ek.size();
+  const size_t bytes = (size_t)ne * kOxP * 16 + (size_t)n_tiles * kOxP * 9 + ((size_t)mats * MM + nV) * 8 +
+                       (nint + kOxParts + 2 + h->M + n_tiles) * sizeof(int) + (size_t)h->M * 8 + 16 * 256;
+  if (bytes > (size_t)256 << 20) {  // leave what the rest of the set-up may need
+    size_t avail = 0, total = 0;
+    CUDA_TRY(cudaMemGetInfo(&avail, &total));
+    if (bytes > avail / 2) return;
+  }
+  unsigned char *p = nullptr;  // one allocation: each costs a small system's set-up some 15 us
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return;
@@ -616,19 +660,25 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
     return q;
   };
   o.x = (long long *)take((size_t)ne * kOxP * 8);
+  o.xt = (long long *)take((size_t)ne * kOxP * 8);
   o.vt = (long long *)take((size_t)n_tiles * kOxP * 8);
   o.dfix = (long long *)take((size_t)mats * MM * 8);
-  if (!h->kpath) o.V = (unsigned long long *)take((size_t)MM * 8);
+  if (nV) o.V = (unsigned long long *)take(nV * 8);
   o.rsh = (signed char *)take((size_t)n_tiles * kOxP);
-  o.ptr = dupload(h, ptr.data(), ptr.size());
-  o.id = dupload(h, id.data(), id.size());
-  o.part = dalloc<int>(h, kOxParts);
-  o.bexp = dalloc<int>(h, 1);
-  o.ee = dalloc<int>(h, h->M);
-  o.ct = dalloc<int>(h, n_tiles);
-  int *d_ek = dupload(h, ek.data(), ek.size());
-  int *d_b = dalloc<int>(h, 1);
-  double *d_s2 = dalloc<double>(h, h->M);
+  o.ptr = (int *)take(nint * sizeof(int));
+  o.id = o.ptr + nptr;
+  const int *d_ek = o.id + id.size();
+  o.part = (int *)take(kOxParts * sizeof(int));
+  o.bexp = (int *)take(sizeof(int));
+  o.ee = (int *)take(h->M * sizeof(int));
+  o.ct = (int *)take(n_tiles * sizeof(int));
+  double *d_s2 = (double *)take(h->M * 8 + sizeof(int));
+  int *d_b = (int *)(d_s2 + h->M);
+  CUDA_TRY(cudaMemsetAsync(d_s2, 0, h->M * 8 + sizeof(int), s));
+  std::vector<int> up(ptr);
+  up.insert(up.end(), id.begin(), id.end());
+  up.insert(up.end(), ek.begin(), ek.end());
+  CUDA_TRY(cudaMemcpyAsync(o.ptr, up.data(), nint * sizeof(int), cudaMemcpyHostToDevice, s));
   Tables tb;
   for (int a = 0; a < 3; ++a) {
     tb.sq[a] = h->d_sq + h->tab_off[a];
@@ -640,16 +690,14 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   CUDA_TRY(cudaGetLastError());
   ox_xmax_kernel<<<1024, 256, 0, s>>>((const double *)o.x, ne * kOxP, d_b);
   CUDA_TRY(cudaGetLastError());
-  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, images ? 9 : 0, d_b, o.x, o.rsh, d_s2);
+  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, images ? 9 : 0, d_b, o.x, o.xt, o.rsh, d_s2);
   CUDA_TRY(cudaGetLastError());
-  std::vector<double> s2(h->M);
-  CUDA_TRY(cudaMemcpy(&o.bX, d_b, sizeof(int), cudaMemcpyDeviceToHost));
-  CUDA_TRY(cudaMemcpy(s2.data(), d_s2, h->M * 8, cudaMemcpyDeviceToHost));
-  dfree(h, d_ek);
-  dfree(h, d_b);
-  dfree(h, d_s2);
+  std::vector<double> s2(h->M + 1);  // (the exponent in the last element's first word)
+  CUDA_TRY(cudaMemcpyAsync(s2.data(), d_s2, h->M * 8 + sizeof(int), cudaMemcpyDeviceToHost, s));
+  CUDA_TRY(cudaStreamSynchronize(s));
+  memcpy(&o.bX, s2.data() + h->M, sizeof(int));
   double mx = 0.0;
-  for (double v : s2) mx = std::max(mx, v);
+  for (int m = 0; m < h->M; ++m) mx = std::max(mx, s2[m]);
   if (o.bX == kOzBad || !std::isfinite(mx)) return;
   o.hexp = ilogb(std::max(mx, 1e-300)) + 1;
   o.geom = geom;
