@@ -29,9 +29,9 @@
 //      bound of |V_ab|, max |v dV| times the largest sum of X^2 of a function
 //      (sums wrap harmlessly in between).
 //
-// One persistent block per SM: warps 0-7 read the accumulators (lane quarter
-// w % 4, column half w / 4), two sets of eight warps cut the digits of the K
-// steps of 16 in turn into a four-stage ring, warp 24 issues the MMAs.  The
+// One persistent block per SM: 8 or 16 warps read the accumulators (lane quarter
+// w % 4, column part w / 4), two or one sets of eight warps cut the digits of
+// the K steps of 16 in turn into a four-stage ring, warp 24 issues the MMAs.  The
 // columns of a tile go in passes of 64 (eight orders of 64 columns fill tensor
 // memory), the last one 64, 32 or 16 wide.  A tile's K is at most 128, one exact
 // chunk.
@@ -42,8 +42,8 @@
 // a step of the set ahead, by lanes along consecutive elements: X is kept twice,
 // [entry][point] for the density and [pair of points][entry] for V, and D is
 // read by its columns.  With one set of builders and V's rows 1 KB apart, D's
-// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.08 and
-// 1.07 ms (11.2 and 9.4 ms on the FP64 pipe).
+// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.03 and
+// 1.00 ms (11.2 and 9.4 ms on the FP64 pipe).
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -64,10 +64,18 @@ constexpr int kOxCols = 64;                     // columns of a pass, at most
 constexpr int kOxA = kOzS * 128 * 32, kOxB = kOzS * kOxCols * 32;
 constexpr int kOxStage = kOxA + kOxB;           // 48 KB
 constexpr int kOxStages = 4;
-constexpr int kOxEpiW = 8, kOxBldW = 8, kOxSets = 2;  // warps: read-out, of a builder set
-constexpr int kOxEpiP = kOxEpiW / 4;            // column parts of the read-out
-constexpr int kOxMmaW = kOxEpiW + kOxSets * kOxBldW;
-constexpr int kOxThreads = (kOxMmaW + 1) * 32;
+constexpr int kOxBldW = 8;                      // warps of a builder set
+constexpr int kOxThreads = 25 * 32;
+// Warps of a pass: the density's builders wait for gathered elements of D, V's
+// read-out has the atomics (16 + 1 x 8 and 8 + 2 x 8 warps, 32 waters: density
+// 1.16 and 1.03 ms, V 1.00 and 1.08 ms)
+template <bool RHO>
+struct OxRoles {
+  static constexpr int epi = RHO ? 8 : 16, sets = RHO ? 2 : 1;
+  static constexpr int parts = epi / 4;               // column parts of the read-out
+  static constexpr int mma = epi + sets * kOxBldW;    // the MMA warp
+  static_assert((mma + 1) * 32 == kOxThreads, "every role has its warps");
+};
 constexpr int kOxParts = 256;                   // partial maxima of a fixed-point conversion
 
 struct OxArgs {
@@ -75,9 +83,9 @@ struct OxArgs {
   KGeom G;                  // lattice offsets (k-points)
   int n_tiles, bX;          // |X| < 2^(bX - 1022)
   const int *ptr, *id;      // entries of a tile; mu, or the image key (k-points)
-  const long long *x;       // [entry][128] (density)
+  const long long *x;       // [entry][128] (density), shifted by rsh
   const long long *xt;      // V: per tile [64 pairs of points][entry][2]
-  const signed char *rsh;   // [tile][128] left shift that fills a point's largest |X|
+  const signed char *rsh;   // [tile][128] left shift that fills 63 bits at a point's largest |X|
   const long long *dfix;    // density: scaled D, or DR per offset
   const int *ee, *ct;       // density: exponents e_a of the functions; -max e_a of a tile
   const int *bexp;          // exponent field of v dV
@@ -153,8 +161,10 @@ __global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     if ((p & 31) == 0) atomicAdd(s2 + (id[e] >> shift), q);
   }
-  // |X| << s stays at most 2^62
-  rsh[(long)t * kOxP + p] = (signed char)(big ? max(0, __clzll((long long)big) - 2) : 0);
+  // X << s fills 63 bits at the point's largest |X|, at most 2^62
+  const int s = big ? max(0, __clzll((long long)big) - 2) : 0;
+  rsh[(long)t * kOxP + p] = (signed char)s;
+  for (int e = ptr[t]; e < ptr[t + 1]; ++e) x[(long)e * kOxP + p] <<= s;
 }
 
 // ---- per evaluation: D and v in fixed point --------------------------------------
@@ -183,12 +193,8 @@ __global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, c
   }
 }
 
-// X_pa 2^e_a in the tile's and the point's scale
-__device__ __forceinline__ long long ox_shift(long long x, int s) {
-  if (s >= 0) return x << s;
-  const int r = min(-s, 62);
-  return (x + (1LL << (r - 1))) >> r;
-}
+// X_pa 2^e_a in the tile's scale, s = max e - e_a (0 to 62)
+__device__ __forceinline__ long long ox_shift(long long x, int s) { return (x + ((1LL << s) >> 1)) >> s; }
 
 // partial maxima of the exponent fields of src
 __global__ void __launch_bounds__(256) ox_max_kernel(const double *src, long n, double scale, int *part) {
@@ -231,8 +237,8 @@ struct OxBars {
   uint64_t part_full[2], part_empty[2];
   uint32_t tbase;
   int stop;
-  __int128 part[2][kOxEpiP - 1][kOxP];  // column parts of rho, two tiles in flight
-  int id[kOxSets * kOxBldW][kOxN], ee[kOxSets * kOxBldW][kOxN];  // entries of a builder warp's tile
+  __int128 part[2][OxRoles<true>::parts - 1][kOxP];  // column parts of rho, two tiles in flight
+  int id[OxRoles<true>::sets * kOxBldW][kOxN], ee[OxRoles<true>::sets * kOxBldW][kOxN];  // entries of a builder warp's tile
 };
 
 // columns of pass h of a tile of n entries: 64, and the last 64, 32 or 16
@@ -292,6 +298,7 @@ __device__ __forceinline__ void ox_mma_step(uint32_t tmem, uint32_t a0, bool fre
 // RHO: density, else V; KP: entries are images, matrices per lattice offset
 template <bool RHO, bool KP>
 __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
+  using W = OxRoles<RHO>;
   extern __shared__ __align__(1024) uint8_t dsm[];
   __shared__ OxBars S;
   const int tid = threadIdx.x, w = uniform(tid >> 5), lane = tid & 31;
@@ -301,9 +308,9 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       mbar_init(&S.empty[s], 1);
     }
     mbar_init(&S.acc_full, 1);
-    mbar_init(&S.acc_empty, kOxEpiW);
+    mbar_init(&S.acc_empty, W::epi);
     for (int q = 0; q < 2; ++q) {
-      mbar_init(&S.part_full[q], kOxEpiW - 4);  // the warps of the parts from 1 up
+      mbar_init(&S.part_full[q], W::epi - 4);  // the warps of the parts from 1 up
       mbar_init(&S.part_empty[q], 4);           // the warps of part 0
     }
     mbar_init(&S.fin, 1);
@@ -319,7 +326,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
   const int M = g.g.M;
   const long MM = (long)M * M;
 
-  if (w == kOxMmaW) {
+  if (w == W::mma) {
     // --------------------------------- MMA issue ---------------------------------
     int fill = 0, ch = 0;
     bool ok = true;
@@ -345,25 +352,25 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
     if (!ok && lane == 0) atomicExch((int *)stop, 1);
     mma_commit(&S.fin);  // every MMA issued has completed before the TMEM is released
     mbar_wait_warp(&S.fin, 0);
-  } else if (w >= kOxEpiW) {
+  } else if (w >= W::epi) {
     // ----------------------------- digits of each K step -----------------------------
     // The inputs of a step are loaded while the previous one's digits are cut
     // (one step's chain of L2 loads is about as long as its MMAs).
     // The sets take the steps in turn.
-    const int bw = w - kOxEpiW, set = bw / kOxBldW, bt = tid - (kOxEpiW + set * kOxBldW) * 32;
+    const int bw = w - W::epi, set = bw / kOxBldW, bt = tid - (W::epi + set * kOxBldW) * 32;
     const int r = bt & 127, hh = bt >> 7;  // A: row, half of the K step
     int first = 0;                         // steps of the tiles before
     bool ok = true;
     for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0, nks = RHO ? (n + 15) / 16 : kOxP / 16;
       const int steps = (n + kOxCols - 1) / kOxCols * nks;
-      const int rs = RHO ? (int)g.rsh[(long)t * kOxP + r] + g.ct[t] : 0;
-      if (RHO) {  // ids and exponents of the tile's entries, a copy per warp
+      if (RHO) {
+        const int top = -g.ct[t];  // ids and exponents of the tile's entries, a copy per warp
         __syncwarp();
         for (int e = lane; e < n; e += 32) {
           const int id = __ldg(g.id + e0 + e);
           S.id[bw][e] = id;
-          S.ee[bw][e] = __ldg(g.ee + (KP ? id >> 9 : id));
+          S.ee[bw][e] = min(top - __ldg(g.ee + (KP ? id >> 9 : id)), 62);
         }
         __syncwarp();
       }
@@ -414,9 +421,9 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       };
       long long xa[8], xb[4];
       longlong2 xv[2];
-      const int st0 = (set + kOxSets - first % kOxSets) % kOxSets;
+      const int st0 = (set + W::sets - first % W::sets) % W::sets;
       if (st0 < steps) load(st0, xa, xb, xv);
-      for (int st = st0; st < steps; st += kOxSets) {
+      for (int st = st0; st < steps; st += W::sets) {
         const int fill = first + st;
         const int h = st / nks, ks = st - h * nks, cw = ox_cols(n, h);
         const int bi = bt & (cw - 1), bq = bt / cw;
@@ -427,7 +434,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int e = ks * 16 + hh * 8 + u;
-          ya[u] = biased(RHO ? (e < n ? ox_shift(xa[u], rs + S.ee[bw][e]) : 0) : xa[u]);
+          ya[u] = biased(RHO ? (e < n ? ox_shift(xa[u], S.ee[bw][e]) : 0) : xa[u]);
         }
         if (RHO) {
 #pragma unroll
@@ -439,7 +446,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
             yb[2 * u + 1] = biased(ox_mul62(xb[2 * u + 1], xv[u].y));
           }
         }
-        if (st + kOxSets < steps) load(st + kOxSets, xa, xb, xv);
+        if (st + W::sets < steps) load(st + W::sets, xa, xb, xv);
         ox_put_all<8>(ya, stg + kstep_off(r, hh * 8), 128 * 32);
         if (bt < cw * 4) ox_put_all<4>(yb, stg + kOxA + kstep_off(bi, bq * 4), cw * 32);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -459,13 +466,13 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0;
       const int gp = RHO ? ox_point(g.g, t, row) : 0;
       const int rs = RHO ? (int)g.rsh[(long)t * kOxP + row] + g.ct[t] : 0;
-      // ids (V) or exponents (density) of the tile's entries, entry lane + 32 q
+      // ids (V) or shifts (density) of the tile's entries, entry lane + 32 q
       int ent[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int e = lane + 32 * q;
         ent[q] = e < n ? __ldg(g.id + e0 + e) : 0;
-        if (RHO && e < n) ent[q] = __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q]));
+        if (RHO && e < n) ent[q] = min(-g.ct[t] - __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q])), 62);
       }
       auto entry = [&](int b) {  // (b: the same in every lane)
         const int lo = b & 32 ? ent[1] : ent[0], hi = b & 32 ? ent[3] : ent[2];
@@ -478,10 +485,10 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) xn[j] = b0 + j < n ? __ldg(g.x + (long)(e0 + b0 + j) * kOxP + row) : 0;
       };
-      if (RHO) ahead(part * (ox_cols(n, 0) / kOxEpiP));
+      if (RHO) ahead(part * (ox_cols(n, 0) / W::parts));
       __int128 acc = 0;
       for (int h = 0; h * kOxCols < n; ++h, ++ch) {
-        const int cw = ox_cols(n, h), cp = cw / kOxEpiP;  // columns of this part
+        const int cw = ox_cols(n, h), cp = cw / W::parts;  // columns of this part
         ok = __all_sync(0xffffffffu, mbar_wait(&S.acc_full, ch & 1, stop));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -490,8 +497,8 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           long long x4[4];
           if (RHO) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) x4[j] = ox_shift(xn[j], rs + entry(b0 + j));
-            const int b1 = c0 + 4 < cp ? b0 + 4 : (h + 1) * kOxCols + part * (ox_cols(n, h + 1) / kOxEpiP);
+            for (int j = 0; j < 4; ++j) x4[j] = ox_shift(xn[j], entry(b0 + j));
+            const int b1 = c0 + 4 < cp ? b0 + 4 : (h + 1) * kOxCols + part * (ox_cols(n, h + 1) / W::parts);
             if (c0 + 4 < cp || (h + 1) * kOxCols < n) ahead(b1);
           }
           uint32_t r[32];
@@ -546,7 +553,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
         }
         ok = __all_sync(0xffffffffu, mbar_wait(&S.part_full[q], (nt >> 1) & 1, stop));
 #pragma unroll
-        for (int c = 0; c < kOxEpiP - 1; ++c) acc += S.part[q][c][row];
+        for (int c = 0; c < W::parts - 1; ++c) acc += S.part[q][c][row];
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.part_empty[q]);
         if (ok && gp >= 0) {
