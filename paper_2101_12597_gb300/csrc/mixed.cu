@@ -573,8 +573,9 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
         // the stage's previous use first (a set may have skipped it): a thread
         // builds one of any three steps in a row, so the copies of the previous
         // ring turn are issued and neither wait can take an older phase for its own
-        if (use > 0 && !mbar_wait(&R.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
-        if (!mbar_wait(&R.tma_full[s], use & 1, stop)) { ok = false; break; }
+        // (voted: a lane that gave up alone would leave the others at the __syncwarp)
+        if (use > 0 && !mbar_wait_warp(&R.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
+        if (!mbar_wait_warp(&R.tma_full[s], use & 1, stop)) { ok = false; break; }
         uint8_t *Bs = dsm + s * kRhoStage + kRhoA;
         const uint8_t *G = Bs + kRhoB;
         const int nrow = max(0, min(kKs, nu - kk * kKs));
@@ -664,11 +665,11 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
       if (lane == 0) mbar_arrive(&R.acc_empty[ab]);
       if (mc == J.a.w - 1) {  // the tile is done: add the column parts
         if (part > 0) {
-          if (ntile > 0) ok = mbar_wait(&R.part_empty, (ntile - 1) & 1, stop);
+          if (ntile > 0) ok = mbar_wait_warp(&R.part_empty, (ntile - 1) & 1, stop);
           R.part[part - 1][pe] = rsum;
           mbar_arrive(&R.part_full);
         } else {
-          ok = mbar_wait(&R.part_full, ntile & 1, stop);
+          ok = mbar_wait_warp(&R.part_full, ntile & 1, stop);
           float2 r = rsum;
 #pragma unroll
           for (int q = 0; q < kRhoParts - 1; ++q) r = df_add(r, R.part[q][pe]);
@@ -907,8 +908,9 @@ __global__ void __launch_bounds__(kVThreads, 1) vmat_tc_kernel(TcBatch B) {
         // before this one's ring turn are issued by now (the job's buffers or
         // the set's last step say so), so the use before the previous one is
         // complete and neither wait can take an older phase for its own.
-        if (use > 0 && !mbar_wait(&R.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
-        if (!mbar_wait(&R.tma_full[s], use & 1, stop)) { ok = false; break; }
+        // (voted: a lane that gave up alone would leave the others at the __syncwarp)
+        if (use > 0 && !mbar_wait_warp(&R.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
+        if (!mbar_wait_warp(&R.tma_full[s], use & 1, stop)) { ok = false; break; }
         uint8_t *Ast = dsm + s * kVStage;
         const uint8_t *Bst = Ast + kVA;
         const int off = kstep_off(b, h * 8);

@@ -428,7 +428,8 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
         const int h = st / nks, ks = st - h * nks, cw = ox_cols(n, h);
         const int bi = bt & (cw - 1), bq = bt / cw;
         const int s = fill % kOxStages, use = fill / kOxStages;
-        if (use > 0 && !mbar_wait(&S.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
+        // (voted: a lane that gave up alone would leave the others at a __syncwarp)
+        if (use > 0 && !mbar_wait_warp(&S.empty[s], (use - 1) & 1, stop)) { ok = false; break; }
         uint8_t *stg = dsm + s * kOxStage;
         unsigned long long ya[8], yb[4];
 #pragma unroll

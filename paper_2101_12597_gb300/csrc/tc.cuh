@@ -82,7 +82,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *b, uint32_t bytes) {
 }
 
 // bounded wait for the completion of the mbarrier phase with parity `parity`;
-// false on timeout or, when `stop` is given, once another role has given up
+// false on timeout or, when `stop` is given, once another role has given up.
+// The lanes of a warp may end it differently: for roles of one lane, or under a
+// vote; a warp that goes on together takes mbar_wait_warp.
 __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity,
                                           const volatile int *stop = nullptr) {
   uint32_t done = 0;
