@@ -367,6 +367,10 @@ constexpr int kRhoEpiW = 16, kRhoBldW = 4;
 constexpr int kRhoParts = kRhoEpiW / 4;  // column parts per lane quarter
 constexpr int kRhoEpi = kRhoEpiW * 32, kRhoBld = kRhoBldW * 32;
 constexpr int kRhoThreads = kRhoEpi + kRhoBld + 64;
+// A builder skips the other set's steps and tells the uses of a stage apart by
+// one parity bit: a step it has built lies at most 3 steps back, and has to
+// lie within the ring (the use before the previous one is then complete)
+static_assert(kRhoStages >= 3, "the builders' parities name one use of a stage");
 
 struct RhoBars {
   uint64_t tma_full[kRhoStages], bld_full[kRhoStages], empty[kRhoStages];
@@ -704,9 +708,9 @@ __global__ void __launch_bounds__(kRhoThreads, 1) rho_tc_kernel(TcBatch B) {
 // its FP32 rounding is 2^-32 of V's scale).  Two accumulator pairs (4 x 128 TMEM
 // columns) alternate between groups, so the read-out of one group overlaps the
 // MMAs of the next.  Warp roles: 0-11 read the accumulators (lane quarter
-// w % 4, every fourth 8-column chunk by w / 4) and add into V by fixed-point
+// w % 4, every third 8-column chunk by w / 4) and add into V by fixed-point
 // reductions; 12-27 build W from the X^T slices and v; 28 streams the X^T
-// slices and the group buffers (v at the points, union entries); 25 issues the
+// slices and the group buffers (v at the points, union entries); 29 issues the
 // MMAs.  Lane i takes the columns j <= i and adds into V[mu_j][mu_i]
 // (mu_j <= mu_i), so a warp's reductions run along a row of V.
 constexpr int kVA = kVSlW * kSlot;  // W slices (128 rows)
@@ -717,6 +721,10 @@ constexpr int kVEpiW = 12, kVBldW = 16;  // warps: 0-11 read-out, 12-27 build W
 constexpr int kVParts = kVEpiW / 4;      // column parts of the read-out per lane quarter
 constexpr int kVEpi = kVEpiW * 32, kVBld = kVBldW * 32;
 constexpr int kVThreads = kVEpi + kVBld + 64;
+// Up to kVBld / 64 builder sets take the steps in turn; a set's last step has to
+// lie within the ring, or the parity it waits for could be an older use's and
+// it would overwrite a stage that the tensor core still reads (no slack: 8, 8)
+static_assert(kVStages >= kVBld / 64, "the builders' parities name one use of a stage");
 // tiles per V group at most (the group size is chosen per handle, <= this):
 // an order-0 accumulator sums kVGmax * 128 products below 2^14 each, so 8
 // keeps every partial sum within 2^24 (exact in FP32)
