@@ -170,9 +170,13 @@ __global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int
 // ---- per evaluation: D and v in fixed point --------------------------------------
 // e with d < 2^2e
 __device__ __forceinline__ int ox_dexp(double d) { return (exp_field(d) - 1021) >> 1; }
+// that of an infinity or NaN: a tile with such a function has no density (where
+// an element of D is not finite, those of its row and column on the diagonal
+// are neither)
+constexpr int kOxBad = (kOzBad - 1021) >> 1;
 
 // D_ab 2^-(e_a + e_b) (one bit in reserve for rounding), the exponents and the
-// tiles' largest ones; diag: the offset 0 of DR (its diagonal bounds every offset)
+// tiles' largest ones (kOxBad: no number); diag: the offset 0 of DR (its diagonal bounds every offset)
 __global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, const double *diag, int M,
                                                       int shift, int n_tiles, const int *ptr, const int *id,
                                                       long long *dst, int *ee, int *ct) {
@@ -467,6 +471,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0;
       const int gp = RHO ? ox_point(g.g, t, row) : 0;
       const int rs = RHO ? (int)g.rsh[(long)t * kOxP + row] + g.ct[t] : 0;
+      const bool bad = RHO && g.ct[t] == -kOxBad;
       // ids (V) or shifts (density) of the tile's entries, entry lane + 32 q
       int ent[4];
 #pragma unroll
@@ -566,7 +571,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           const int drop = max(0, 65 - lz);
           const double m = (double)(long long)(unsigned long long)(u >> drop);
           const double v = oz_scale(m, drop + 2 * g.bX - 2152 - 2 * rs);
-          g.rho[gp] = neg ? -v : v;
+          g.rho[gp] = bad ? nan("") : neg ? -v : v;
         }
       }
     }
