@@ -24,9 +24,9 @@ namespace etdm {
 
 constexpr int kTriBits = 200;  // sections end at 2^-kTriBits of the block's norm
 
-// the smallest e^2 of a scaled block (|T| < 1): a smaller off-diagonal counts
-// as 2^-400, so that two minors in a row never vanish together
-constexpr double kTriE2Min = 0x1p-800;
+// the smallest e^2 of a scaled block (|T| < 1): a smaller off-diagonal counts as
+// 2^-210, below what the sections resolve
+constexpr double kTriE2Min = 0x1p-420;
 
 ETDM_HD long long tri_bits(double v) {
   long long b;
@@ -40,45 +40,43 @@ ETDM_HD double tri_double(long long b) {
 }
 ETDM_HD int tri_exp(double v) { return (int)((tri_bits(v) >> 52) & 0x7ff); }
 
-// v 2^k by the exponent field, k such that it stays below 2^1000; zero where
-// it leaves the normal range
+// v 2^k by the exponent field, k such that it stays below 2^1000; a zero of its
+// sign where it leaves the normal range
 ETDM_HD double tri_shift(double v, int k) {
   const int f = tri_exp(v);
-  return f > 0 && f + k > 0 ? tri_double(tri_bits(v) + ((long long)k << 52)) : 0.0;
+  const long long b = tri_bits(v);
+  return tri_double(f > 0 && f + k > 0 ? b + ((long long)k << 52) : b & (1LL << 63));
 }
 
 // Eigenvalues of rows [p, q) below x (block scaled to |T| < 1, |x| < 1.1;
 // kTriE2Min <= e2 <= 1): the signs of the leading principal minors p_j =
 // (d_j - x) p_(j-1) - e_(j-1)^2 p_(j-2), a change of sign per eigenvalue below
-// x; a zero counts as the sign opposite to its predecessor.  Three FP64
-// operations per row (the quotient form divides), with the exponents kept in
-// range by integer operations: whenever the larger of the two minors leaves
-// 2^+-100, both are shifted to bring it to 1.  A row grows them by at most 4,
-// and of two rows the larger shrinks by no less than 2^-800; a minor lost to
-// the range lies 2^-900 below its neighbour.
+// x (a zero's sign does not matter: its neighbours have opposite ones, and
+// either way one change falls on the two rows).  Three FP64 operations per row
+// (the quotient form divides).  Every second row, minors that have left
+// 2^+-100 are shifted by their exponents to bring the larger of the last two to
+// 1: a row grows them by at most 4 and shrinks the larger by no less than
+// 2^-422, so they stay in range wherever x lies, also far below the norm
+// (every eighth row was not enough there), and two in a row never vanish.
 ETDM_HD int tri_count(const double *d, const double *e2, int p, int q, double x) {
-  auto neg = [](double v, int before) {  // sign bit, a zero's from its predecessor
-    const long long b = tri_bits(v);
-    return (b << 1) == 0 ? !before : (int)((unsigned long long)b >> 63);
+  auto changes = [](double v, double w) {  // of sign, 0 or 1
+    return (int)((unsigned long long)(tri_bits(v) ^ tri_bits(w)) >> 63);
   };
   double pm = 1.0, pc = d[p] - x;
-  int s = neg(pc, 0), c = s, em = 1023;
-  for (int j = p + 1; j < q; ++j) {
-    int ec = tri_exp(pc);
-    const int top = ec > em ? ec : em;
+  int c = changes(pm, pc), j = p + 1;
+  for (; j + 1 < q; j += 2) {
+    const double p1 = fma(d[j] - x, pc, -(e2[j - 1] * pm));
+    const double p2 = fma(d[j + 1] - x, p1, -(e2[j] * pc));
+    c += changes(pc, p1) + changes(p1, p2);
+    pm = p1;
+    pc = p2;
+    const int em = tri_exp(pm), ec = tri_exp(pc), top = ec > em ? ec : em;
     if ((unsigned)(top - 923) > 200u) {
       pc = tri_shift(pc, 1023 - top);
       pm = tri_shift(pm, 1023 - top);
-      ec = tri_exp(pc);
     }
-    const double pn = fma(d[j] - x, pc, -(e2[j - 1] * pm));
-    pm = pc;
-    em = ec;
-    pc = pn;
-    const int t = neg(pc, s);
-    c += t != s;
-    s = t;
   }
+  if (j < q) c += changes(pc, fma(d[j] - x, pc, -(e2[j - 1] * pm)));
   return c;
 }
 
