@@ -296,12 +296,11 @@ struct OxGrid {
   GridGeom geom{};
   int n_tiles = 0;
   bool images = false;          // entries are images (k-points), else functions
-  int bX = 0, hexp = 0;         // exponents of X and of V's fixed point
   int *ptr = nullptr, *id = nullptr;
   long long *x = nullptr, *xt = nullptr, *vt = nullptr, *dfix = nullptr;
   unsigned long long *V = nullptr;
-  signed char *rsh = nullptr;
-  int *part = nullptr, *bexp = nullptr, *ee = nullptr, *ct = nullptr;
+  short *pexp = nullptr, *q = nullptr;
+  int *part = nullptr, *bexp = nullptr, *vq = nullptr, *hx = nullptr, *ee = nullptr, *ct = nullptr;
 };
 
 }  // namespace etdm

@@ -16,18 +16,24 @@
 //      reach the tile summed (the phase between images is 1 at the Gamma point;
 //      a box of 6.4 A has some 150 images of 16 functions per tile); with
 //      k-points one entry per image, the pair's lattice offset looked up.
-//      Evaluated once in FP64 at set-up and kept as fixed point, [entry][128].
+//      Evaluated once in FP64 at set-up and kept twice, with all of its 53 bits:
+//      for the density, whose rows are points, as a left-justified mantissa and
+//      its distance from the point's largest exponent, [entry][128]; for V, whose
+//      rows are entries, in fixed point with the power of two of the entry's
+//      largest value in the tile.  (One power of two for the whole system left
+//      the density around a molecule, where X is 1e-16 of the largest, with
+//      relative errors of 2e-2; now 2e-14.)
 //   D: positive semidefinite, so |D_ab| <= sqrt(D_aa D_bb): D_ab 2^-(e_a + e_b)
 //      with D_aa < 2^2e_a in fixed point, and X_pa shifted by e_a in the density
 //      pass.  Where the density is faint because its functions' D is, it keeps
 //      its relative accuracy, which rho^(1/3) passes on to v (one power of two
 //      for all of D left 1e-9 of v, and 6e-11 of H, on an atom whose orbitals
 //      are empty).
-//   v: fixed point with the power of two of its largest element; 62 bits below
-//      it are nine more than FP64 keeps of it.
+//   v: fixed point with the power of two of its largest element in the tile.
 //   V: 64-bit fixed point with a factor 2 in reserve over the Cauchy-Schwarz
-//      bound of |V_ab|, max |v dV| times the largest sum of X^2 of a function
-//      (sums wrap harmlessly in between).
+//      bound of |V_ab|, max |v dV| (sum X_a^2 sum X_b^2)^(1/2) (sums wrap
+//      harmlessly in between): the unit is 2^-62 of that bound, where an FP64
+//      sum rounds at 2^-53 of the terms it adds.
 //
 // One persistent block per SM: 8 or 16 warps read the accumulators (lane quarter
 // w % 4, column part w / 4), two or one sets of eight warps cut the digits of
@@ -42,8 +48,9 @@
 // a step of the set ahead, by lanes along consecutive elements: X is kept twice,
 // [entry][point] for the density and [pair of points][entry] for V, and D is
 // read by its columns.  With one set of builders and V's rows 1 KB apart, D's
-// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.03 and
-// 1.00 ms (11.2 and 9.4 ms on the FP64 pipe).
+// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.06 and
+// 1.03 ms (11.2 and 9.4 ms on the FP64 pipe), of which the exponents of single
+// values and of entries and tiles take 0.02 and 0.04.
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -67,8 +74,8 @@ constexpr int kOxStages = 4;
 constexpr int kOxBldW = 8;                      // warps of a builder set
 constexpr int kOxThreads = 25 * 32;
 // Warps of a pass: the density's builders wait for gathered elements of D, V's
-// read-out has the atomics (16 + 1 x 8 and 8 + 2 x 8 warps, 32 waters: density
-// 1.16 and 1.03 ms, V 1.00 and 1.08 ms)
+// read-out has the atomics (16 + 1 x 8 and 8 + 2 x 8 warps, 32 waters, with one
+// power of two for X: density 1.16 and 1.03 ms, V 1.00 and 1.08 ms)
 template <bool RHO>
 struct OxRoles {
   static constexpr int epi = RHO ? 8 : 16, sets = RHO ? 2 : 1;
@@ -81,18 +88,19 @@ constexpr int kOxParts = 256;                   // partial maxima of a fixed-poi
 struct OxArgs {
   GridGeom g;               // 4 x 4 x 8 tiles
   KGeom G;                  // lattice offsets (k-points)
-  int n_tiles, bX;          // |X| < 2^(bX - 1022)
+  int n_tiles;
   const int *ptr, *id;      // entries of a tile; mu, or the image key (k-points)
-  const long long *x;       // [entry][128] (density), shifted by rsh
-  const long long *xt;      // V: per tile [64 pairs of points][entry][2]
-  const signed char *rsh;   // [tile][128] left shift that fills 63 bits at a point's largest |X|
+  const long long *x;       // density: [entry][128] words of ox_word
+  const long long *xt;      // V: per tile [64 pairs of points][entry][2], fixed point
+  const short *pexp;        // density: [tile][128] exponent field of a point's largest |X|
+  const short *q;           // V: [entry] bits from the entry's unit to the function's
   const long long *dfix;    // density: scaled D, or DR per offset
   const int *ee, *ct;       // density: exponents e_a of the functions; -max e_a of a tile
   const int *bexp;          // exponent field of v dV
   double *rho;
   const long long *vt;      // V: v dV in tile order
+  const int *vq;            // V: [tile] bits from the tile's unit of v to the largest
   unsigned long long *V;    // V: sums, [M][M] (upper triangle), or [offset][M][M]
-  int sh;                   // V: left shift (right when negative) of a tile's sum
   int full;                 // V: both triangles
   int *flags;
 };
@@ -112,17 +120,23 @@ __device__ __forceinline__ int ox_ridx(const KGeom &G, int ka, int kb) {
 }
 
 // ---- set-up -------------------------------------------------------------------
-// X of a tile's entries in FP64 (into the fixed-point table's memory): entry e
-// sums the images keys[ek[e]] .. keys[ek[e + 1] - 1]
-__global__ void __launch_bounds__(kOxP) ox_basis_kernel(GridGeom g, Tables tb, const int *ptr,
-                                                        const int *ek, const int *keys, double *x) {
-  const int t = blockIdx.x, p = threadIdx.x;
+// X of a tile's entries in FP64 (into the tables' memory): entry e sums the
+// images keys[ek[e]] .. keys[ek[e + 1] - 1]; the exponent fields of a point's
+// and of an entry's largest |X| in the tile, and sum X^2 per function
+__global__ void __launch_bounds__(kOxP) ox_basis_kernel(GridGeom g, Tables tb, const int *ptr, const int *id,
+                                                        int shift, const int *ek, const int *keys, double *x,
+                                                        short *pexp, short *xe, double *s2) {
+  __shared__ int big[kOxN];
+  const int t = blockIdx.x, p = threadIdx.x, e0 = ptr[t], n = ptr[t + 1] - e0;
   const int bz = t % g.nbz, by = (t / g.nbz) % g.nby, bx = t / (g.nbz * g.nby);
   const int i = bx * 4 + (p >> 5), j = by * 4 + ((p >> 3) & 3), k = bz * 8 + (p & 7);
   const bool in = i < g.nx && j < g.ny && k < g.nz;
-  for (int e = ptr[t]; e < ptr[t + 1]; ++e) {
+  big[p] = 1;
+  __syncthreads();
+  int top = 1;
+  for (int e = 0; e < n; ++e) {
     double s = 0.0;
-    for (int q = ek[e]; in && q < ek[e + 1]; ++q) {
+    for (int q = ek[e0 + e]; in && q < ek[e0 + e + 1]; ++q) {
       const int key = keys[q], mu = key >> 9;
       const int ix = ((key >> 6) & 7) - 4 + kImgMax, iy = ((key >> 3) & 7) - 4 + kImgMax,
                 iz = (key & 7) - 4 + kImgMax;
@@ -131,40 +145,60 @@ __global__ void __launch_bounds__(kOxP) ox_basis_kernel(GridGeom g, Tables tb, c
       const double r2 = __dadd_rn(__dadd_rn(tb.sq[0][ax], tb.sq[1][ay]), tb.sq[2][az]);
       if (r2 < tb.rc2[mu]) s += tb.norm[mu] * tb.ex[0][ax] * tb.ex[1][ay] * tb.ex[2][az];
     }
-    x[(long)e * kOxP + p] = s;
-  }
-}
-
-// largest exponent field of x into *bmax
-__global__ void __launch_bounds__(256) ox_xmax_kernel(const double *x, long n, int *bmax) {
-  int m = 1;
-  for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x)
-    m = max(m, exp_field(x[e]));
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0) atomicMax(bmax, m);
-}
-
-// FP64 -> fixed point in place, the points' shifts, and sum X^2 per function
-__global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int *id, int shift,
-                                                       const int *bmax, long long *x,
-                                                       long long *xt, signed char *rsh, double *s2) {
-  const int t = blockIdx.x, p = threadIdx.x, b = *bmax, n = ptr[t + 1] - ptr[t];
-  long long *const xp = xt + (long)ptr[t] * kOxP + (long)(p >> 1) * n * 2 + (p & 1);
-  unsigned long long big = 0;
-  for (int e = ptr[t]; e < ptr[t + 1]; ++e) {
-    const double v = __longlong_as_double(x[(long)e * kOxP + p]);
-    const long long f = to_fixed(v, b);
-    x[(long)e * kOxP + p] = f;
-    xp[2 * (e - ptr[t])] = f;
-    big = max(big, (unsigned long long)(f < 0 ? -f : f));
-    double q = v * v;
+    x[(long)(e0 + e) * kOxP + p] = s;
+    const int f = exp_field(s), m = __reduce_max_sync(0xffffffffu, f);
+    top = max(top, f);
+    double q = s * s;
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    if ((p & 31) == 0) atomicAdd(s2 + (id[e] >> shift), q);
+    if ((p & 31) == 0) {
+      atomicMax(&big[e], m);
+      atomicAdd(s2 + (id[e0 + e] >> shift), q);
+    }
   }
-  // X << s fills 63 bits at the point's largest |X|, at most 2^62
-  const int s = big ? max(0, __clzll((long long)big) - 2) : 0;
-  rsh[(long)t * kOxP + p] = (signed char)s;
-  for (int e = ptr[t]; e < ptr[t + 1]; ++e) x[(long)e * kOxP + p] <<= s;
+  pexp[(long)t * kOxP + p] = (short)top;
+  __syncthreads();
+  if (p < n) xe[e0 + p] = (short)big[p];
+}
+
+// X as a left-justified mantissa (53 bits, 2^61 <= |m| < 2^62) and, in its lowest
+// seven bits, the distance k of its exponent field from the point's largest,
+// top: X = m 2^(top - 1084 - k).  Zero 63 bits below the largest, and for
+// subnormal numbers (their squares are no FP64 numbers).
+__device__ __forceinline__ long long ox_word(double v, int top) {
+  const long long b = __double_as_longlong(v);
+  const int f = exp_field(v), k = top - f;
+  if (f == 0 || k > 63) return 0;
+  const long long m = ((b & 0xfffffffffffffLL) | (1LL << 52)) << 9;
+  return (b < 0 ? -m : m) | k;
+}
+// its fixed-point value in the unit 2^(top - 1084 + s), s = 0 to 63
+__device__ __forceinline__ long long ox_value(long long w, int s) {
+  const int r = min(s + ((int)w & 127), 63);
+  return ((w & ~511LL) + (long long)((1ULL << r) >> 1)) >> r;
+}
+
+// h with sum X^2 < 2^2h for a function's sum of squares
+__device__ __forceinline__ int ox_hexp(double s2) { return (max(exp_field(s2), 1) - 1021) >> 1; }
+
+// the tables of X (x holds it in FP64 on entry), and the entries' exponent
+// fields q as the bits from their units to those of their functions
+__global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int *id, int shift, int M,
+                                                       const short *pexp, const double *s2, long long *x,
+                                                       long long *xt, short *q, int *hx) {
+  __shared__ short xe[kOxN];
+  const int t = blockIdx.x, p = threadIdx.x, e0 = ptr[t], n = ptr[t + 1] - e0;
+  if (p < n) xe[p] = q[e0 + p];
+  __syncthreads();
+  if (p < n)  // at least 0: X^2 <= sum X^2; a unit 100 bits away adds nothing
+    q[e0 + p] = (short)min(ox_hexp(s2[id[e0 + p] >> shift]) - xe[p] + 1022, 100);
+  const int top = pexp[(long)t * kOxP + p];
+  long long *const xp = xt + (long)e0 * kOxP + (long)(p >> 1) * n * 2 + (p & 1);
+  for (int e = 0; e < n; ++e) {
+    const double v = __longlong_as_double(x[(long)(e0 + e) * kOxP + p]);
+    xp[2 * e] = to_fixed(v, xe[e]);
+    x[(long)(e0 + e) * kOxP + p] = ox_word(v, top);
+  }
+  for (int m = blockIdx.x * kOxP + p; m < M; m += gridDim.x * kOxP) hx[m] = ox_hexp(s2[m]);
 }
 
 // ---- per evaluation: D and v in fixed point --------------------------------------
@@ -197,9 +231,6 @@ __global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, c
   }
 }
 
-// X_pa 2^e_a in the tile's scale, s = max e - e_a (0 to 62)
-__device__ __forceinline__ long long ox_shift(long long x, int s) { return (x + ((1LL << s) >> 1)) >> s; }
-
 // partial maxima of the exponent fields of src
 __global__ void __launch_bounds__(256) ox_max_kernel(const double *src, long n, double scale, int *part) {
   __shared__ int sm[8];
@@ -224,14 +255,25 @@ __device__ __forceinline__ int ox_total_max(const int *part, int np) {
   for (int q = 1; q < 8; ++q) m = max(m, sm[q]);
   return m;
 }
-// v dV in tile order (0 outside the grid)
-__global__ void __launch_bounds__(256) ox_vfix_kernel(GridGeom g, int n_tiles, const double *v,
-                                                      const int *part, int np, long long *dst, int *bexp) {
-  const int b = ox_total_max(part, np);
+// v dV in tile order (0 outside the grid), a warp per tile, in the unit of the
+// tile's largest; vq: the bits from there to the largest of all
+__global__ void __launch_bounds__(256) ox_vfix_kernel(GridGeom g, int n_tiles, const double *v, const int *part,
+                                                      int np, long long *dst, int *vq, int *bexp) {
+  const int b = ox_total_max(part, np), lane = threadIdx.x & 31;
   if (blockIdx.x == 0 && threadIdx.x == 0) *bexp = b;
-  for (long q = (long)blockIdx.x * 256 + threadIdx.x; q < (long)n_tiles * kOxP; q += (long)gridDim.x * 256) {
-    const int gp = ox_point(g, (int)(q / kOxP), (int)(q % kOxP));
-    dst[q] = (gp < 0 || b == kOzBad) ? 0 : to_fixed(v[gp] * g.dV, b);
+  for (long t = ((long)blockIdx.x * 256 + threadIdx.x) >> 5; t < n_tiles; t += gridDim.x * 8L) {
+    double x[4];
+    int m = 1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int gp = ox_point(g, (int)t, lane + 32 * u);
+      x[u] = gp < 0 ? 0.0 : v[gp] * g.dV;
+      m = max(m, exp_field(x[u]));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) vq[t] = min(b - m, 100);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) dst[t * kOxP + lane + 32 * u] = b == kOzBad ? 0 : to_fixed(x[u], m);
   }
 }
 
@@ -374,7 +416,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
         for (int e = lane; e < n; e += 32) {
           const int id = __ldg(g.id + e0 + e);
           S.id[bw][e] = id;
-          S.ee[bw][e] = min(top - __ldg(g.ee + (KP ? id >> 9 : id)), 62);
+          S.ee[bw][e] = min(top - __ldg(g.ee + (KP ? id >> 9 : id)), 63);
         }
         __syncwarp();
       }
@@ -439,7 +481,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int e = ks * 16 + hh * 8 + u;
-          ya[u] = biased(RHO ? (e < n ? ox_shift(xa[u], S.ee[bw][e]) : 0) : xa[u]);
+          ya[u] = biased(RHO ? (e < n ? ox_value(xa[u], S.ee[bw][e]) : 0) : xa[u]);
         }
         if (RHO) {
 #pragma unroll
@@ -470,21 +512,26 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
     for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++nt) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0;
       const int gp = RHO ? ox_point(g.g, t, row) : 0;
-      const int rs = RHO ? (int)g.rsh[(long)t * kOxP + row] + g.ct[t] : 0;
+      const int rexp = RHO ? (int)g.pexp[(long)t * kOxP + row] - g.ct[t] : 0;
       const bool bad = RHO && g.ct[t] == -kOxBad;
-      // ids (V) or shifts (density) of the tile's entries, entry lane + 32 q
+      // ids and, from bit 24, units (V) or shifts (density) of the tile's entries,
+      // entry lane + 32 q
       int ent[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int e = lane + 32 * q;
         ent[q] = e < n ? __ldg(g.id + e0 + e) : 0;
-        if (RHO && e < n) ent[q] = min(-g.ct[t] - __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q])), 62);
+        if (RHO && e < n) ent[q] = min(-g.ct[t] - __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q])), 63);
+        if (!RHO && e < n) ent[q] |= (int)__ldg(g.q + e0 + e) << 24;
       }
       auto entry = [&](int b) {  // (b: the same in every lane)
         const int lo = b & 32 ? ent[1] : ent[0], hi = b & 32 ? ent[3] : ent[2];
         return __shfl_sync(0xffffffffu, b & 64 ? hi : lo, b & 31);
       };
-      const int ida = RHO ? 0 : ent[quad];  // entry `row`
+      const int ida = RHO ? 0 : ent[quad] & 0xffffff;  // entry `row`
+      // bits from the unit of the tile's sums to V's, without the column's; at
+      // least 6 (2^-1084 x 2^-1084 x 2^56 against 2^(-1084 - 1022))
+      const int ra = RHO ? 0 : 6 + (ent[quad] >> 24) + __ldg(g.vq + t);
       // density: X of the next four columns, loaded a group ahead
       long long xn[4];
       auto ahead = [&](int b0) {
@@ -503,7 +550,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           long long x4[4];
           if (RHO) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) x4[j] = ox_shift(xn[j], entry(b0 + j));
+            for (int j = 0; j < 4; ++j) x4[j] = ox_value(xn[j], entry(b0 + j));
             const int b1 = c0 + 4 < cp ? b0 + 4 : (h + 1) * kOxCols + part * (ox_cols(n, h + 1) / W::parts);
             if (c0 + 4 < cp || (h + 1) * kOxCols < n) ahead(b1);
           }
@@ -518,7 +565,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int b = b0 + j;
-            const int idb = RHO ? 0 : entry(b);
+            const int eb = RHO ? 0 : entry(b), idb = eb & 0xffffff;
             long long hi = 0, lo = 0;
             oz_add(r, j, hi, lo);
             const __int128 T = ((__int128)hi << 32) + lo;  // |T| <= 2^75
@@ -526,8 +573,8 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
               // (a column beyond n has X = 0)
               acc += ((__int128)(long long)(T >> 13) * x4[j]) >> 8;
             } else if (b < n && b <= row && row < n) {
-              const long long v = g.sh >= 0 ? (long long)(T << g.sh)
-                                            : (long long)((T + ((__int128)1 << (-g.sh - 1))) >> -g.sh);
+              const int r = min(ra + (eb >> 24), 100);
+              const long long v = (long long)((T + ((__int128)1 << (r - 1))) >> r);
               if (v != 0) {
                 if (KP) {  // VR[n_a - n_b][mu_a][mu_b], and the transposed pair
                   const int ri = ox_ridx(g.G, ida, idb);
@@ -570,7 +617,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           const int lz = top ? __clzll((long long)top) : 64 + __clzll((long long)(unsigned long long)u);
           const int drop = max(0, 65 - lz);
           const double m = (double)(long long)(unsigned long long)(u >> drop);
-          const double v = oz_scale(m, drop + 2 * g.bX - 2152 - 2 * rs);
+          const double v = oz_scale(m, drop + 2 * rexp - 2152);
           g.rho[gp] = bad ? nan("") : neg ? -v : v;
         }
       }
@@ -583,23 +630,25 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
   if (tid == 0 && S.stop) atomicExch(g.flags + FLAG_ERR, ETDM_ERR_TIMEOUT);
 }
 
-// H += the fixed-point sums (upper triangle), unit 2^(bV + hexp - 1084)
-__global__ void __launch_bounds__(256) ox_vadd_kernel(const unsigned long long *V, int M, int hexp,
+// H += the fixed-point sums (upper triangle), unit 2^(bV + h_a + h_b - 1084)
+__global__ void __launch_bounds__(256) ox_vadd_kernel(const unsigned long long *V, int M, const int *hx,
                                                       const int *bexp, double *H) {
   const int b = *bexp;
   const long MM = (long)M * M;
   for (long e = (long)blockIdx.x * 256 + threadIdx.x; e < MM; e += (long)gridDim.x * 256) {
-    if (e / M > e % M) continue;
-    H[e] += b == kOzBad ? nan("") : oz_scale((double)(long long)V[e], b + hexp - 1084);
+    const int i = (int)(e / M), j = (int)(e % M);
+    if (i > j) continue;
+    H[e] += b == kOzBad ? nan("") : oz_scale((double)(long long)V[e], b + hx[i] + hx[j] - 1084);
   }
 }
-// the sums as FP64, in place
-__global__ void __launch_bounds__(256) ox_vcvt_kernel(double *V, long n, int hexp, const int *bexp) {
+// the sums as FP64, in place (a matrix per blockIdx.y)
+__global__ void __launch_bounds__(256) ox_vcvt_kernel(double *V, int M, const int *hx, const int *bexp) {
   const int b = *bexp;
-  for (long e = (long)blockIdx.x * 256 + threadIdx.x; e < n; e += (long)gridDim.x * 256) {
-    const long long q = __double_as_longlong(V[e]);
-    V[e] = b == kOzBad ? nan("") : oz_scale((double)q, b + hexp - 1084);
-  }
+  const unsigned e = blockIdx.x * 256 + threadIdx.x, MM = (unsigned)M * M;
+  if (e >= MM) return;
+  const int h = hx[e / (unsigned)M] + hx[e % (unsigned)M];
+  double *const v = V + (size_t)blockIdx.y * MM + e;
+  *v = b == kOzBad ? nan("") : oz_scale((double)__double_as_longlong(*v), b + h - 1084);
 }
 
 // ---- host side -------------------------------------------------------------------
@@ -611,9 +660,8 @@ OxArgs ox_args(etdm_handle *h) {
   a.g = o.geom;
   a.G = h->kg;
   a.n_tiles = o.n_tiles;
-  a.bX = o.bX;
-  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.xt = o.xt; a.rsh = o.rsh;
-  a.dfix = o.dfix; a.ee = o.ee; a.ct = o.ct; a.bexp = o.bexp; a.vt = o.vt;
+  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.xt = o.xt; a.pexp = o.pexp; a.q = o.q;
+  a.dfix = o.dfix; a.ee = o.ee; a.ct = o.ct; a.bexp = o.bexp; a.vt = o.vt; a.vq = o.vq;
   a.flags = h->d_flags;
   return a;
 }
@@ -634,8 +682,8 @@ int ox_parts(long n) { return (int)std::max<long>(1, std::min<long>(kOxParts, (n
 // Tables of the passes from the 4 x 4 x 8 tiles' image lists (ptr, keys on the
 // host and on the device).  `images`: one entry per image, else per function.
 // Leaves h->ox.n_tiles = 0 (the passes of grid.cu run) when a tile has more
-// than 128 entries or the tables (2 KB per entry) would take more than half of
-// the free memory.
+// than 128 entries, the tables (2 KB per entry) would take more than half of
+// the free memory, or a function has no finite sum of squares.
 void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vector<int> &kptr,
               const std::vector<int> &keys, const int *d_keys, bool images, cudaStream_t s) {
   OxGrid &o = h->ox;
@@ -650,12 +698,13 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
     if (ptr[t + 1] - ptr[t] > kOxN) return;
   }
   const long ne = (long)id.size();
-  if (ne == 0) return;
+  if (ne == 0 || h->M >= (images ? 1 << 15 : 1 << 24)) return;  // (ids share a word with 8 bits)
   ek.push_back((int)keys.size());
   const long mats = images ? h->kg.nR : 1, MM = (long)h->M * h->M;
   const size_t nptr = ptr.size(), nV = h->kpath ? 0 : (size_t)MM, nint = nptr + id.size() + ek.size();
-  const size_t bytes = (size_t)ne * kOxP * 16 + (size_t)n_tiles * kOxP * 9 + ((size_t)mats * MM + nV) * 8 +
-                       (nint + kOxParts + 2 + h->M + n_tiles) * sizeof(int) + (size_t)h->M * 8 + 16 * 256;
+  const size_t bytes = (size_t)ne * (kOxP * 16 + 2) + (size_t)n_tiles * kOxP * 10 +
+                       ((size_t)mats * MM + nV) * 8 + (nint + kOxParts + 1 + 2 * h->M + 2 * n_tiles) * sizeof(int) +
+                       (size_t)h->M * 8 + 16 * 256;
   if (bytes > (size_t)256 << 20) {  // leave what the rest of the set-up may need
     size_t avail = 0, total = 0;
     CUDA_TRY(cudaMemGetInfo(&avail, &total));
@@ -677,17 +726,19 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   o.vt = (long long *)take((size_t)n_tiles * kOxP * 8);
   o.dfix = (long long *)take((size_t)mats * MM * 8);
   if (nV) o.V = (unsigned long long *)take(nV * 8);
-  o.rsh = (signed char *)take((size_t)n_tiles * kOxP);
+  o.pexp = (short *)take((size_t)n_tiles * kOxP * sizeof(short));
+  o.q = (short *)take((size_t)ne * sizeof(short));
   o.ptr = (int *)take(nint * sizeof(int));
   o.id = o.ptr + nptr;
   const int *d_ek = o.id + id.size();
   o.part = (int *)take(kOxParts * sizeof(int));
   o.bexp = (int *)take(sizeof(int));
   o.ee = (int *)take(h->M * sizeof(int));
+  o.hx = (int *)take(h->M * sizeof(int));
   o.ct = (int *)take(n_tiles * sizeof(int));
-  double *d_s2 = (double *)take(h->M * 8 + sizeof(int));
-  int *d_b = (int *)(d_s2 + h->M);
-  CUDA_TRY(cudaMemsetAsync(d_s2, 0, h->M * 8 + sizeof(int), s));
+  o.vq = (int *)take(n_tiles * sizeof(int));
+  double *d_s2 = (double *)take(h->M * 8);
+  CUDA_TRY(cudaMemsetAsync(d_s2, 0, h->M * 8, s));
   std::vector<int> up(ptr);
   up.insert(up.end(), id.begin(), id.end());
   up.insert(up.end(), ek.begin(), ek.end());
@@ -699,20 +750,17 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   }
   tb.norm = h->d_norm;
   tb.rc2 = h->d_rc2;
-  ox_basis_kernel<<<n_tiles, kOxP, 0, s>>>(geom, tb, o.ptr, d_ek, d_keys, (double *)o.x);
+  const int shift = images ? 9 : 0;
+  ox_basis_kernel<<<n_tiles, kOxP, 0, s>>>(geom, tb, o.ptr, o.id, shift, d_ek, d_keys, (double *)o.x, o.pexp,
+                                           o.q, d_s2);
   CUDA_TRY(cudaGetLastError());
-  ox_xmax_kernel<<<1024, 256, 0, s>>>((const double *)o.x, ne * kOxP, d_b);
+  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, shift, h->M, o.pexp, d_s2, o.x, o.xt, o.q, o.hx);
   CUDA_TRY(cudaGetLastError());
-  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, images ? 9 : 0, d_b, o.x, o.xt, o.rsh, d_s2);
-  CUDA_TRY(cudaGetLastError());
-  std::vector<double> s2(h->M + 1);  // (the exponent in the last element's first word)
-  CUDA_TRY(cudaMemcpyAsync(s2.data(), d_s2, h->M * 8 + sizeof(int), cudaMemcpyDeviceToHost, s));
+  std::vector<double> s2(h->M);
+  CUDA_TRY(cudaMemcpyAsync(s2.data(), d_s2, h->M * 8, cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  memcpy(&o.bX, s2.data() + h->M, sizeof(int));
-  double mx = 0.0;
-  for (int m = 0; m < h->M; ++m) mx = std::max(mx, s2[m]);
-  if (o.bX == kOzBad || !std::isfinite(mx)) return;
-  o.hexp = ilogb(std::max(mx, 1e-300)) + 1;
+  for (double v : s2)
+    if (!std::isfinite(v)) return;
   o.geom = geom;
   o.images = images;
   o.n_tiles = n_tiles;
@@ -739,14 +787,13 @@ cudaError_t ox_vmat(etdm_handle *h, const double *v, unsigned long long *V, bool
   const OxGrid &o = h->ox;
   const int np = ox_parts(h->G);
   ox_max_kernel<<<np, 256, 0, s>>>(v, h->G, o.geom.dV, o.part);
-  ox_vfix_kernel<<<(int)std::min<long>(4 * h->num_sms, ((long)o.n_tiles * kOxP + 255) / 256), 256, 0, s>>>(
-      o.geom, o.n_tiles, v, o.part, np, o.vt, o.bexp);
+  ox_vfix_kernel<<<(int)std::min<long>(8 * h->num_sms, ((long)o.n_tiles + 7) / 8), 256, 0, s>>>(
+      o.geom, o.n_tiles, v, o.part, np, o.vt, o.vq, o.bexp);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   OxArgs a = ox_args(h);
   a.V = V;
   a.full = full;
-  a.sh = 2 * o.bX - o.hexp - 2050;
   return o.images ? ox_launch<false, true>(a, h->num_sms, s) : ox_launch<false, false>(a, h->num_sms, s);
 }
 }  // namespace
@@ -758,7 +805,7 @@ cudaError_t launch_ox_vmat(etdm_handle *h, const double *v, double *H, cudaStrea
   cudaError_t e = cudaMemsetAsync(o.V, 0, MM * 8, s);
   if (e != cudaSuccess) return e;
   if ((e = ox_vmat(h, v, o.V, false, s)) != cudaSuccess) return e;
-  ox_vadd_kernel<<<(int)std::min<long>(4 * h->num_sms, (MM + 255) / 256), 256, 0, s>>>(o.V, h->M, o.hexp, o.bexp, H);
+  ox_vadd_kernel<<<(int)std::min<long>(4 * h->num_sms, (MM + 255) / 256), 256, 0, s>>>(o.V, h->M, o.hx, o.bexp, H);
   return cudaGetLastError();
 }
 
@@ -769,7 +816,8 @@ cudaError_t launch_ox_vmat_k(etdm_handle *h, const double *v, double *VR, cudaSt
   cudaError_t e = cudaMemsetAsync(VR, 0, n * 8, s);
   if (e != cudaSuccess) return e;
   if ((e = ox_vmat(h, v, (unsigned long long *)VR, true, s)) != cudaSuccess) return e;
-  ox_vcvt_kernel<<<(int)std::min<long>(8 * h->num_sms, (n + 255) / 256), 256, 0, s>>>(VR, n, o.hexp, o.bexp);
+  const unsigned bx = (unsigned)(((long)h->M * h->M + 255) / 256);
+  ox_vcvt_kernel<<<dim3(bx, h->kg.nR), 256, 0, s>>>(VR, h->M, o.hx, o.bexp);
   return cudaGetLastError();
 }
 
