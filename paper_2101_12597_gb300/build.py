@@ -17,7 +17,7 @@ SOURCES = ["capi.cu", "dense.cu", "grid.cu", "potential.cu", "mixed.cu", "fftdf.
            "plan.cu", "batch.cu", "kpoint.cu", "kpath.cu",
            "ozgemm.cu", "ozgrid.cu"]
 HEADERS = ["internal.h", "device.cuh", "host.h", "pair.cuh", "linesearch.h", "tc.cuh", "kpoint.h",
-           "ozdigits.cuh", "tcgemm.cuh", "dense_small.cuh", "tridiag.h"]
+           "ozdigits.cuh", "tcgemm.cuh", "dense_small.cuh", "tridiag.h", "roots.h"]
 NVCC = os.environ.get("NVCC", "nvcc")
 FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo",
          "-std=c++17", "--extended-lambda", "-Xcompiler", "-fPIC"]
