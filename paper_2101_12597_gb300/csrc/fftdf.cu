@@ -529,11 +529,12 @@ DfLaunch df_launch_plan(const std::vector<DfArgs> &args) {
 template <bool BIG>
 static cudaError_t df_potential(const DfLaunch &L, const DfArgs *av, const int *active,
                                 cudaStream_t s) {
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(zfwd_kernel<BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smz)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(zinv_pot_kernel<BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smz)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(yfft_kernel<BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smy)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(xpois_kernel<BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smx)) != cudaSuccess) return e;
+  // 8 lines of kMaxFFT points take more than 16 of the 79 that still have 16
+  constexpr int most = (kMaxFFT + 2 * 8 * kMaxFFT) * (int)sizeof(float4);
+  static_assert(kZPairs == 8 && 79 + 2 * 16 * 79 <= kMaxFFT + 2 * 8 * kMaxFFT, "the largest launch");
+  for (auto k : {zfwd_kernel<BIG>, zinv_pot_kernel<BIG>, xpois_kernel<BIG>})
+    if (const cudaError_t e = allow_smem(k, most)) return e;
+  if (const cudaError_t e = allow_smem(yfft_kernel<BIG>, most)) return e;
   zfwd_kernel<BIG><<<dim3(L.zb, L.n_sys), kDfThreads, L.smz, s>>>(av, active);
   yfft_kernel<BIG><<<dim3(L.yb, L.n_sys), kDfThreads, L.smy, s>>>(av, active, -1);
   xpois_kernel<BIG><<<dim3(L.xb, L.n_sys), kDfThreads, L.smx, s>>>(av, active);

@@ -382,8 +382,7 @@ static size_t rho_smem(int n) {
 cudaError_t launch_rho_fp64(etdm_handle *h, const double *D, double *rho, cudaStream_t s) {
   if (h->ox.n_tiles) return launch_ox_rho(h, D, rho, s);
   size_t sm = rho_smem(h->max_list);
-  cudaError_t e = cudaFuncSetAttribute(rho_fp64_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = allow_smem(rho_fp64_kernel, (int)rho_smem(kMaxList));
   if (e != cudaSuccess) return e;
   rho_fp64_kernel<<<h->n_tiles, kRhoThreads, sm, s>>>(h->geom, tables_of(h), h->d_tile_ptr,
                                                       h->d_keys, D, rho);
@@ -449,11 +448,12 @@ __global__ void __launch_bounds__(kRhoThreads) vmat_fp64_kernel(GridGeom g, Tabl
   }
 }
 
+static size_t vmat_smem(int n) { return (size_t)n * (kTP + 1) * 16 + (size_t)n * 4 + 16; }
+
 cudaError_t launch_vmat_fp64(etdm_handle *h, const double *v, double *Hacc, cudaStream_t s) {
   if (h->ox.n_tiles) return launch_ox_vmat(h, v, Hacc, s);
-  size_t sm = (size_t)h->max_list * (kTP + 1) * 16 + (size_t)h->max_list * 4 + 16;
-  cudaError_t e = cudaFuncSetAttribute(vmat_fp64_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  size_t sm = vmat_smem(h->max_list);
+  cudaError_t e = allow_smem(vmat_fp64_kernel, (int)vmat_smem(kMaxList));
   if (e != cudaSuccess) return e;
   vmat_fp64_kernel<<<h->n_tiles, kRhoThreads, sm, s>>>(h->geom, tables_of(h), h->d_tile_ptr,
                                                        h->d_keys, v, Hacc);
@@ -528,16 +528,15 @@ __global__ void __launch_bounds__(kRhoThreads) rho_k_kernel(GridGeom g, Tables t
 cudaError_t launch_rho_k(etdm_handle *h, const double *DR, double *rho, cudaStream_t s) {
   if (h->ox.n_tiles) return launch_ox_rho(h, DR, rho, s);
   size_t sm = rho_smem(h->max_list) + (size_t)h->max_list * 4;
-  cudaError_t e = cudaFuncSetAttribute(rho_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
+  cudaError_t e = allow_smem(rho_k_kernel, (int)rho_smem(kMaxList) + kMaxList * 4);
   if (e != cudaSuccess) return e;
   rho_k_kernel<<<h->n_tiles, kRhoThreads, sm, s>>>(h->geom, tables_of(h), h->d_tile_ptr,
                                                    h->d_keys, h->kg, DR, rho);
   return cudaGetLastError();
 }
 
-// VR[R][mu_a][mu_b] (zeroed by the launcher) += dV sum_p X_ap v_p X_bp for every ordered pair of list
-// entries (computed once per unordered pair).
+// VR[R][mu_a][mu_b] (zeroed by the launcher) += dV sum_p X_ap v_p X_bp for every
+// ordered pair of list entries (computed once per unordered pair).
 __global__ void __launch_bounds__(kRhoThreads) vmat_k_kernel(GridGeom g, Tables tb,
                                                              const int *tile_ptr,
                                                              const int *keys, KGeom G,
@@ -602,11 +601,10 @@ __global__ void __launch_bounds__(kRhoThreads) vmat_k_kernel(GridGeom g, Tables 
 
 cudaError_t launch_vmat_k(etdm_handle *h, const double *v, double *VR, cudaStream_t s) {
   if (h->ox.n_tiles) return launch_ox_vmat_k(h, v, VR, s);
-  size_t sm = (size_t)h->max_list * (kTP + 1) * 16 + (size_t)h->max_list * 8 + 16;
+  size_t sm = vmat_smem(h->max_list) + (size_t)h->max_list * 4;
   cudaError_t e = cudaMemsetAsync(VR, 0, (size_t)h->kg.nR * h->M * h->M * 8, s);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(vmat_k_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
+  e = allow_smem(vmat_k_kernel, (int)vmat_smem(kMaxList) + kMaxList * 4);
   if (e != cudaSuccess) return e;
   vmat_k_kernel<<<h->n_tiles, kRhoThreads, sm, s>>>(h->geom, tables_of(h), h->d_tile_ptr,
                                                     h->d_keys, h->kg, v, VR);

@@ -509,6 +509,13 @@ cudaError_t launch_vmat_fp64(etdm_handle *h, const double *v, double *Hacc, cuda
 cudaError_t launch_ox_rho(etdm_handle *h, const double *D, double *rho, cudaStream_t s);
 cudaError_t launch_ox_vmat(etdm_handle *h, const double *v, double *H, cudaStream_t s);
 cudaError_t launch_ox_vmat_k(etdm_handle *h, const double *v, double *VR, cudaStream_t s);
+// Dynamic shared memory that launches of a kernel may take: a constant of the
+// kernel.  The attribute belongs to the kernel, not to a launch, so a size of
+// this call's would refuse the launch of another host thread with a larger one.
+template <class... A>
+cudaError_t allow_smem(void (*kernel)(A...), int bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
 // fft and potential (potential.cu)
 cudaError_t launch_twiddles(etdm_handle *h, cudaStream_t s);
 cudaError_t fft3d(etdm_handle *h, double2 *data, int sign, cudaStream_t s);

@@ -204,8 +204,7 @@ cudaError_t fft3d(etdm_handle *h, double2 *data, int sign, cudaStream_t s) {
     long blocks = (Bd == 1) ? (A + kFftLines - 1) / kFftLines
                             : A * ((Bd + kFftLines - 1) / kFftLines);
     size_t sm = (size_t)2 * kFftLines * n * sizeof(double2);
-    cudaError_t e = cudaFuncSetAttribute(fft_axis_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_smem(fft_axis_kernel, 2 * kFftLines * kMaxFFT * (int)sizeof(double2));
     if (e != cudaSuccess) return e;
     fft_axis_kernel<<<(unsigned)blocks, kFftThreads, sm, s>>>(data, A, Bd, h->d_tw + tw_off[ax],
                                                               plan, sign);
@@ -541,14 +540,10 @@ cudaError_t launch_potential(etdm_handle *h, const double *rho, double *v, doubl
   const int bz = pot_lines(pairs, h->num_sms), by = pot_lines(ly, h->num_sms), bx = pot_lines(lx, h->num_sms);
   auto smem = [](int n, int lb) { return (size_t)(n + 2 * lb * n) * sizeof(double2); };
   const size_t sz = smem(a.nz, bz), sy = smem(a.ny, by), sx = smem(a.nx, bx);
-  cudaError_t e;
-  auto attr = [&e](auto k, size_t sm) {
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    return e == cudaSuccess;
-  };
-  if (!attr(pot_zfwd_kernel, sz) || !attr(pot_y_kernel, sy) || !attr(pot_x_kernel, sx) ||
-      !attr(pot_zinv_kernel<false>, sz) || !attr(pot_zinv_kernel<true>, sz))
-    return e;
+  const int most = (int)smem(kMaxFFT, kPotLinesMax);
+  for (auto k : {pot_zfwd_kernel, pot_x_kernel, pot_zinv_kernel<false>, pot_zinv_kernel<true>})
+    if (const cudaError_t e = allow_smem(k, most)) return e;
+  if (const cudaError_t e = allow_smem(pot_y_kernel, most)) return e;
   const unsigned gz = (unsigned)((pairs + bz - 1) / bz), gy = (unsigned)((ly + by - 1) / by),
                  gx = (unsigned)((lx + bx - 1) / bx);
   a.lines = bz;
