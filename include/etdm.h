@@ -341,7 +341,13 @@ int etdm_get_array(etdm_handle *h, int32_t which, void *host_dst,
  * elapsed milliseconds since the last call into ms[ETDM_NSTAGES] and the
  * number of timed launches of each stage into counts[ETDM_NSTAGES]; the last
  * entry of counts is the number of kernel launches issued since the last
- * call. */
+ * call.  It also tells which kernels a handle runs: the FP64 grid passes take
+ * tables of the basis on the grid (2 KB per function and 128-point tile, at
+ * set-up, after everything that a handle cannot do without, and at most half
+ * of the memory that is then free unless they are below 256 MB) where no tile
+ * has more than 128 functions (with k-points: images); a density is then 2
+ * launches and a potential matrix 4, without the tables 1 each, with the same
+ * results to rounding. */
 enum {
   ETDM_STAGE_DENSE_FWD = 0, /* exp(A), O = C0 U, D (cooperative kernel) */
   ETDM_STAGE_RHO = 1,       /* basis -> grid density */

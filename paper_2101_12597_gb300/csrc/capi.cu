@@ -389,7 +389,14 @@ void etdm::setup_ox(etdm_handle *h, bool images, cudaStream_t s) {
   long n = 0;
   const GridGeom geom = make_geom(h, 4, 4, 8, &T);
   std::vector<int> ptr;
-  build_lists(h, geom, T, &d_ptr, &d_keys, &n, &max_list, INT32_MAX, s, &ptr);
+  try {
+    build_lists(h, geom, T, &d_ptr, &d_keys, &n, &max_list, INT32_MAX, s, &ptr);
+  } catch (const Fail &f) {  // without memory for the lists there are no tables
+    dfree(h, d_ptr);
+    dfree(h, d_keys);
+    if (f.code != ETDM_ERR_OOM) throw;
+    return;
+  }
   std::vector<int> keys(n);
   if (n > 0) CUDA_TRY(cudaMemcpy(keys.data(), d_keys, n * sizeof(int), cudaMemcpyDeviceToHost));
   ox_setup(h, geom, T, ptr, keys, d_keys, images, s);
@@ -611,7 +618,6 @@ void init_impl(etdm_handle *h, const etdm_system *sys, const etdm_options *opt) 
   CUDA_TRY(fft3d(h, h->d_fft, +1, s));
   CUDA_TRY(launch_real_part(h, h->d_fft, h->d_vext, s));
   if (h->precision == ETDM_PREC_MIXED) CUDA_TRY(launch_df_setup(h, s));  // twiddles, v_ext, Poisson kernel
-  if (h->precision == ETDM_PREC_FP64 && !h->kpath) setup_ox(h, false, s);
   if (h->kpath) {  // full A over k-points: its own matrices and reference
     h->d_E = dalloc<double>(h, 2);
     h->d_eterms = dalloc<double>(h, 4);
@@ -683,12 +689,16 @@ void init_impl(etdm_handle *h, const etdm_system *sys, const etdm_options *opt) 
   etdm::alloc_opt_buffers(h);
 
   // reference orbitals: Loewdin S^(-1/2), columns by ascending diag of C0^T h_core C0
+  double *d_diag = dalloc<double>(h, M);
+  int *d_perm = dalloc<int>(h, M);
+  double *d_tmpC = dalloc<double>(h, MM);
   inverse_sqrt(h, s);
+  // (optional memory last: what a set-up cannot do without has been allocated)
+  if (h->precision == ETDM_PREC_FP64) setup_ox(h, false, s);
   CUDA_TRY(cudaMemcpyAsync(h->d_H, h->d_T, MM * 8, cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(launch_vmat_fp64(h, h->d_vext, h->d_H, s));
   symmetrize_upper_kernel<<<256, 256, 0, s>>>(h->d_H, M);
   CUDA_TRY(cudaGetLastError());
-  double *d_diag = dalloc<double>(h, M);
   CUDA_TRY(launch_diag_quad(h->d_C0, h->d_H, d_diag, M, s));
   std::vector<double> diag(M);
   CUDA_TRY(cudaMemcpy(diag.data(), d_diag, M * 8, cudaMemcpyDeviceToHost));
@@ -698,9 +708,7 @@ void init_impl(etdm_handle *h, const etdm_system *sys, const etdm_options *opt) 
   std::iota(h->order.begin(), h->order.end(), 0);
   std::stable_sort(h->order.begin(), h->order.end(),
                    [&](int x, int y) { return diag[x] < diag[y]; });
-  int *d_perm = dalloc<int>(h, M);
   CUDA_TRY(cudaMemcpy(d_perm, h->order.data(), M * sizeof(int), cudaMemcpyHostToDevice));
-  double *d_tmpC = dalloc<double>(h, MM);
   CUDA_TRY(cudaMemcpyAsync(d_tmpC, h->d_C0, MM * 8, cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(launch_permute_cols(d_tmpC, d_perm, h->d_C0, M, s));
   if (h->precision == ETDM_PREC_MIXED) {  // the mixed path's dense chains run on float pairs

@@ -62,17 +62,6 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
     G.Rm[a] = std::min(2 * kImgMax, (int)floor(2.0 * rmax / h->L[a]) + 1);
     G.nR *= 2 * G.Rm[a] + 1;
   }
-  // the FP64 grid passes on the tensor cores; at the Gamma point alone every
-  // offset has phase 1, so one real-space matrix and merged images suffice
-  bool gamma = true;
-  for (double x : h->h_kfrac) gamma = gamma && x == 0.0;
-  const KGeom table = G;
-  if (gamma) {
-    G.Rm[0] = G.Rm[1] = G.Rm[2] = 0;
-    G.nR = 1;
-  }
-  setup_ox(h, !gamma, s);
-  if (!h->ox.n_tiles) G = table;
   h->d_kfrac = dupload(h, h->h_kfrac.data(), 3 * (size_t)nk);
   h->d_kw = dupload(h, h->h_kw.data(), (size_t)nk);
   G.kfrac = h->d_kfrac;
@@ -110,6 +99,28 @@ void init_kpoints(etdm_handle *h, const etdm_system *sys) {
     h->d_kfro = dalloc<double>(h, 2 * k_fro2_parts());
   }
 
+  // Optional memory last: what a set-up cannot do without has been allocated.
+  // The FP64 grid passes on the tensor cores; at the Gamma point alone every
+  // offset has phase 1, so one real-space matrix and merged images suffice
+  bool gamma = true;
+  for (double x : h->h_kfrac) gamma = gamma && x == 0.0;
+  const KGeom table = G;
+  if (gamma) {
+    G.Rm[0] = G.Rm[1] = G.Rm[2] = 0;
+    G.nR = 1;
+  }
+  setup_ox(h, !gamma, s);
+  if (!h->ox.n_tiles) {
+    G = table;
+  } else if (gamma) {
+    CUDA_TRY(k_phases(G, phase, s));  // (1, the first in the table's place)
+    if ((size_t)table.nR * MM * 8 > (size_t)64 << 20) {
+      for (double **p : {&h->d_kDR, &h->d_kVR}) {
+        dfree(h, *p);
+        *p = dalloc<double>(h, MM);
+      }
+    }
+  }
   if (oz_takes(M, nk)) oz_alloc(h, M, nk);
 
   // S(k), T(k); h_core(k) = T(k) + V_ext(k)
