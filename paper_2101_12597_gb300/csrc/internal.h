@@ -300,6 +300,7 @@ struct OxGrid {
   long long *x = nullptr, *xt = nullptr, *vt = nullptr, *dfix = nullptr;
   unsigned long long *V = nullptr;
   short *pexp = nullptr, *q = nullptr;
+  uint8_t *kx = nullptr, *pmin = nullptr;
   int *part = nullptr, *bexp = nullptr, *vq = nullptr, *hx = nullptr, *ee = nullptr, *ct = nullptr;
 };
 

@@ -24,11 +24,12 @@
 //      the density around a molecule, where X is 1e-16 of the largest, with
 //      relative errors of 2e-2; now 2e-14.)
 //   D: positive semidefinite, so |D_ab| <= sqrt(D_aa D_bb): D_ab 2^-(e_a + e_b)
-//      with D_aa < 2^2e_a in fixed point, and X_pa shifted by e_a in the density
-//      pass.  Where the density is faint because its functions' D is, it keeps
-//      its relative accuracy, which rho^(1/3) passes on to v (one power of two
-//      for all of D left 1e-9 of v, and 6e-11 of H, on an atom whose orbitals
-//      are empty).
+//      with D_aa < 2^2e_a in fixed point, and X_pa 2^e_a in the density pass,
+//      in fixed point with the power of two of the point's largest of these.
+//      Where the density is faint it keeps its relative accuracy, which
+//      rho^(1/3) passes on to v (one power of two for all of D left 1e-9 of v,
+//      and 6e-11 of H, on an atom whose orbitals are empty; one per tile 1e-12
+//      and 3e-13).
 //   v: fixed point with the power of two of its largest element in the tile.
 //   V: 64-bit fixed point with a factor 2 in reserve over the Cauchy-Schwarz
 //      bound of |V_ab|, max |v dV| (sum X_a^2 sum X_b^2)^(1/2) (sums wrap
@@ -48,9 +49,10 @@
 // a step of the set ahead, by lanes along consecutive elements: X is kept twice,
 // [entry][point] for the density and [pair of points][entry] for V, and D is
 // read by its columns.  With one set of builders and V's rows 1 KB apart, D's
-// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.06 and
+// 2 KB, a step waited for its loads: 32 waters 1.23 and 1.21 ms, now 1.07 and
 // 1.03 ms (11.2 and 9.4 ms on the FP64 pipe), of which the exponents of single
-// values and of entries and tiles take 0.02 and 0.04.
+// values and of entries and tiles take 0.04 each; the points' shifts take another
+// 0.02 with the conversion of D.
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -93,6 +95,7 @@ struct OxArgs {
   const long long *x;       // density: [entry][128] words of ox_word
   const long long *xt;      // V: per tile [64 pairs of points][entry][2], fixed point
   const short *pexp;        // density: [tile][128] exponent field of a point's largest |X|
+  const uint8_t *pmin;      // density: [tile][128] bits from max |X_pa| max 2^e_a to max |X_pa 2^e_a|
   const short *q;           // V: [entry] bits from the entry's unit to the function's
   const long long *dfix;    // density: scaled D, or DR per offset
   const int *ee, *ct;       // density: exponents e_a of the functions; -max e_a of a tile
@@ -162,18 +165,18 @@ __global__ void __launch_bounds__(kOxP) ox_basis_kernel(GridGeom g, Tables tb, c
 
 // X as a left-justified mantissa (53 bits, 2^61 <= |m| < 2^62) and, in its lowest
 // seven bits, the distance k of its exponent field from the point's largest,
-// top: X = m 2^(top - 1084 - k).  Zero 63 bits below the largest, and for
+// top: X = m 2^(top - 1084 - k).  Zero 128 bits below the largest, and for
 // subnormal numbers (their squares are no FP64 numbers).
 __device__ __forceinline__ long long ox_word(double v, int top) {
   const long long b = __double_as_longlong(v);
   const int f = exp_field(v), k = top - f;
-  if (f == 0 || k > 63) return 0;
+  if (f == 0 || k > 127) return 0;
   const long long m = ((b & 0xfffffffffffffLL) | (1LL << 52)) << 9;
   return (b < 0 ? -m : m) | k;
 }
-// its fixed-point value in the unit 2^(top - 1084 + s), s = 0 to 63
+// its fixed-point value in the unit 2^(top - 1084 + s), s + k >= 0 unless it is zero
 __device__ __forceinline__ long long ox_value(long long w, int s) {
-  const int r = min(s + ((int)w & 127), 63);
+  const int r = min(max(s + ((int)w & 127), 0), 63);
   return ((w & ~511LL) + (long long)((1ULL << r) >> 1)) >> r;
 }
 
@@ -184,7 +187,7 @@ __device__ __forceinline__ int ox_hexp(double s2) { return (max(exp_field(s2), 1
 // fields q as the bits from their units to those of their functions
 __global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int *id, int shift, int M,
                                                        const short *pexp, const double *s2, long long *x,
-                                                       long long *xt, short *q, int *hx) {
+                                                       long long *xt, uint8_t *kx, short *q, int *hx) {
   __shared__ short xe[kOxN];
   const int t = blockIdx.x, p = threadIdx.x, e0 = ptr[t], n = ptr[t + 1] - e0;
   if (p < n) xe[p] = q[e0 + p];
@@ -196,7 +199,9 @@ __global__ void __launch_bounds__(kOxP) ox_xfix_kernel(const int *ptr, const int
   for (int e = 0; e < n; ++e) {
     const double v = __longlong_as_double(x[(long)(e0 + e) * kOxP + p]);
     xp[2 * e] = to_fixed(v, xe[e]);
-    x[(long)(e0 + e) * kOxP + p] = ox_word(v, top);
+    const long long w = ox_word(v, top);
+    x[(long)(e0 + e) * kOxP + p] = w;
+    kx[(long)(e0 + e) * kOxP + p] = w ? (uint8_t)(w & 127) : 255;
   }
   for (int m = blockIdx.x * kOxP + p; m < M; m += gridDim.x * kOxP) hx[m] = ox_hexp(s2[m]);
 }
@@ -210,10 +215,11 @@ __device__ __forceinline__ int ox_dexp(double d) { return (exp_field(d) - 1021) 
 constexpr int kOxBad = (kOzBad - 1021) >> 1;
 
 // D_ab 2^-(e_a + e_b) (one bit in reserve for rounding), the exponents and the
-// tiles' largest ones (kOxBad: no number); diag: the offset 0 of DR (its diagonal bounds every offset)
+// tiles' largest ones (kOxBad: no number), the points' shifts pmin; diag: the offset 0 of DR (its diagonal bounds every offset)
 __global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, const double *diag, int M,
                                                       int shift, int n_tiles, const int *ptr, const int *id,
-                                                      long long *dst, int *ee, int *ct) {
+                                                      const uint32_t *kx, long long *dst, int *ee, int *ct,
+                                                      uint32_t *pmin) {
   const long MM = (long)M * M, gtid = (long)blockIdx.x * 256 + threadIdx.x, gs = (long)gridDim.x * 256;
   for (long q = gtid; q < n; q += gs) {
     const long r = q % MM;
@@ -223,11 +229,35 @@ __global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, c
   for (long a = gtid; a < M; a += gs) ee[a] = ox_dexp(diag[a * (M + 1)]);
   const int lane = threadIdx.x & 31;
   for (long t = gtid >> 5; t < n_tiles; t += gs >> 5) {
-    int m = -2000;
-    for (int e = ptr[t] + lane; e < ptr[t + 1]; e += 32)
-      m = max(m, ox_dexp(diag[(long)(id[e] >> shift) * (M + 1)]));
+    const int e0 = ptr[t], n = ptr[t + 1] - e0;
+    int ex[4], m = -2000;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = lane + 32 * q;
+      ex[q] = e < n ? ox_dexp(diag[(long)(id[e0 + e] >> shift) * (M + 1)]) : -2000;
+      m = max(m, ex[q]);
+    }
     m = __reduce_max_sync(0xffffffffu, m);
     if (lane == 0) ct[t] = -m;
+    // four points a lane, in 16-bit pairs: the least k + (max e - e_a) over the
+    // entries, 255 at most (32 entries' loads in flight)
+    uint32_t least[2] = {0x00ff00ffu, 0x00ff00ffu};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (32 * q >= n) break;
+      uint32_t k4[32];
+#pragma unroll
+      for (int l = 0; l < 32; ++l)
+        k4[l] = 32 * q + l < n ? __ldg(kx + (long)(e0 + 32 * q + l) * 32 + lane) : 0xffffffffu;
+      const uint32_t d = min(m - ex[q], 255) * 0x00010001u;
+#pragma unroll
+      for (int l = 0; l < 32; ++l) {
+        const uint32_t dl = __shfl_sync(0xffffffffu, d, l);
+        least[0] = __viaddmin_u16x2(__byte_perm(k4[l], 0, 0x4140), dl, least[0]);
+        least[1] = __viaddmin_u16x2(__byte_perm(k4[l], 0, 0x4342), dl, least[1]);
+      }
+    }
+    pmin[t * 32 + lane] = __byte_perm(least[0], least[1], 0x6420);
   }
 }
 
@@ -410,13 +440,15 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
     for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0, nks = RHO ? (n + 15) / 16 : kOxP / 16;
       const int steps = (n + kOxCols - 1) / kOxCols * nks;
+      int rm = 0;
       if (RHO) {
         const int top = -g.ct[t];  // ids and exponents of the tile's entries, a copy per warp
+        rm = g.pmin[(long)t * kOxP + r];
         __syncwarp();
         for (int e = lane; e < n; e += 32) {
           const int id = __ldg(g.id + e0 + e);
           S.id[bw][e] = id;
-          S.ee[bw][e] = min(top - __ldg(g.ee + (KP ? id >> 9 : id)), 63);
+          S.ee[bw][e] = min(top - __ldg(g.ee + (KP ? id >> 9 : id)), 512);
         }
         __syncwarp();
       }
@@ -481,7 +513,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int e = ks * 16 + hh * 8 + u;
-          ya[u] = biased(RHO ? (e < n ? ox_value(xa[u], S.ee[bw][e]) : 0) : xa[u]);
+          ya[u] = biased(RHO ? (e < n ? ox_value(xa[u], S.ee[bw][e] - rm) : 0) : xa[u]);
         }
         if (RHO) {
 #pragma unroll
@@ -512,7 +544,8 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
     for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++nt) {
       const int e0 = g.ptr[t], n = g.ptr[t + 1] - e0;
       const int gp = RHO ? ox_point(g.g, t, row) : 0;
-      const int rexp = RHO ? (int)g.pexp[(long)t * kOxP + row] - g.ct[t] : 0;
+      const int rm = RHO ? (int)g.pmin[(long)t * kOxP + row] : 0;
+      const int rexp = RHO ? (int)g.pexp[(long)t * kOxP + row] - g.ct[t] - rm : 0;
       const bool bad = RHO && g.ct[t] == -kOxBad;
       // ids and, from bit 24, units (V) or shifts (density) of the tile's entries,
       // entry lane + 32 q
@@ -521,7 +554,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
       for (int q = 0; q < 4; ++q) {
         const int e = lane + 32 * q;
         ent[q] = e < n ? __ldg(g.id + e0 + e) : 0;
-        if (RHO && e < n) ent[q] = min(-g.ct[t] - __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q])), 63);
+        if (RHO && e < n) ent[q] = min(-g.ct[t] - __ldg(g.ee + (KP ? ent[q] >> 9 : ent[q])), 512);
         if (!RHO && e < n) ent[q] |= (int)__ldg(g.q + e0 + e) << 24;
       }
       auto entry = [&](int b) {  // (b: the same in every lane)
@@ -550,7 +583,7 @@ __global__ void __launch_bounds__(kOxThreads, 1) ox_pass_kernel(OxArgs g) {
           long long x4[4];
           if (RHO) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) x4[j] = ox_value(xn[j], entry(b0 + j));
+            for (int j = 0; j < 4; ++j) x4[j] = ox_value(xn[j], entry(b0 + j) - rm);
             const int b1 = c0 + 4 < cp ? b0 + 4 : (h + 1) * kOxCols + part * (ox_cols(n, h + 1) / W::parts);
             if (c0 + 4 < cp || (h + 1) * kOxCols < n) ahead(b1);
           }
@@ -660,7 +693,8 @@ OxArgs ox_args(etdm_handle *h) {
   a.g = o.geom;
   a.G = h->kg;
   a.n_tiles = o.n_tiles;
-  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.xt = o.xt; a.pexp = o.pexp; a.q = o.q;
+  a.ptr = o.ptr; a.id = o.id; a.x = o.x; a.xt = o.xt; a.pexp = o.pexp; a.pmin = o.pmin;
+  a.q = o.q;
   a.dfix = o.dfix; a.ee = o.ee; a.ct = o.ct; a.bexp = o.bexp; a.vt = o.vt; a.vq = o.vq;
   a.flags = h->d_flags;
   return a;
@@ -682,7 +716,7 @@ int ox_parts(long n) { return (int)std::max<long>(1, std::min<long>(kOxParts, (n
 // Tables of the passes from the 4 x 4 x 8 tiles' image lists (ptr, keys on the
 // host and on the device).  `images`: one entry per image, else per function.
 // Leaves h->ox.n_tiles = 0 (the passes of grid.cu run) when a tile has more
-// than 128 entries, the tables (2 KB per entry) would take more than half of
+// than 128 entries, the tables (2.1 KB per entry) would take more than half of
 // the free memory, or a function has no finite sum of squares.
 void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vector<int> &kptr,
               const std::vector<int> &keys, const int *d_keys, bool images, cudaStream_t s) {
@@ -702,9 +736,9 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   ek.push_back((int)keys.size());
   const long mats = images ? h->kg.nR : 1, MM = (long)h->M * h->M;
   const size_t nptr = ptr.size(), nV = h->kpath ? 0 : (size_t)MM, nint = nptr + id.size() + ek.size();
-  const size_t bytes = (size_t)ne * (kOxP * 16 + 2) + (size_t)n_tiles * kOxP * 10 +
+  const size_t bytes = (size_t)ne * (kOxP * 17 + 2) + (size_t)n_tiles * kOxP * 11 +
                        ((size_t)mats * MM + nV) * 8 + (nint + kOxParts + 1 + 2 * h->M + 2 * n_tiles) * sizeof(int) +
-                       (size_t)h->M * 8 + 16 * 256;
+                       (size_t)h->M * 8 + 20 * 256;
   if (bytes > (size_t)256 << 20) {  // leave what the rest of the set-up may need
     size_t avail = 0, total = 0;
     CUDA_TRY(cudaMemGetInfo(&avail, &total));
@@ -728,6 +762,8 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   if (nV) o.V = (unsigned long long *)take(nV * 8);
   o.pexp = (short *)take((size_t)n_tiles * kOxP * sizeof(short));
   o.q = (short *)take((size_t)ne * sizeof(short));
+  o.kx = take((size_t)ne * kOxP);
+  o.pmin = take((size_t)n_tiles * kOxP);
   o.ptr = (int *)take(nint * sizeof(int));
   o.id = o.ptr + nptr;
   const int *d_ek = o.id + id.size();
@@ -754,7 +790,8 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
   ox_basis_kernel<<<n_tiles, kOxP, 0, s>>>(geom, tb, o.ptr, o.id, shift, d_ek, d_keys, (double *)o.x, o.pexp,
                                            o.q, d_s2);
   CUDA_TRY(cudaGetLastError());
-  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, shift, h->M, o.pexp, d_s2, o.x, o.xt, o.q, o.hx);
+  ox_xfix_kernel<<<n_tiles, kOxP, 0, s>>>(o.ptr, o.id, shift, h->M, o.pexp, d_s2, o.x, o.xt, o.kx, o.q,
+                                          o.hx);
   CUDA_TRY(cudaGetLastError());
   std::vector<double> s2(h->M);
   CUDA_TRY(cudaMemcpyAsync(s2.data(), d_s2, h->M * 8, cudaMemcpyDeviceToHost, s));
@@ -773,7 +810,7 @@ cudaError_t launch_ox_rho(etdm_handle *h, const double *D, double *rho, cudaStre
   const long work = std::max(n, (long)o.n_tiles * 32);
   ox_dfix_kernel<<<(int)std::min<long>(8 * h->num_sms, (work + 255) / 256), 256, 0, s>>>(
       D, n, D + (o.images ? (h->kg.nR - 1) / 2 : 0) * (long)h->M * h->M, h->M, o.images ? 9 : 0, o.n_tiles,
-      o.ptr, o.id, o.dfix, o.ee, o.ct);
+      o.ptr, o.id, (const uint32_t *)o.kx, o.dfix, o.ee, o.ct, (uint32_t *)o.pmin);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   OxArgs a = ox_args(h);

@@ -88,3 +88,45 @@ def test_crystal_density_relative_to_its_terms(kmesh):
     print(f"kmesh={kmesh}: {err:.1e}, smallest {mag.min() / mag.max():.1e}")
     assert mag.min() < 1e-6 * mag.max() and err <= TOL
     s.close()
+
+
+@pytest.mark.parametrize("exps", [(2.0, 8.0), (0.8, 3.0)])
+def test_potential_over_atoms_without_electrons(exps):
+    """Half of a row of atoms holds no electron, and A = 0, so the density there is
+    of the tails of the others' orbitals (1e-8 to 1e-40 of the largest), in tiles
+    that also list occupied functions.  rho^(1/3) passes its relative error on:
+    rho to 1e-11 of its terms as above, H to 64 roundings of its largest element
+    (v to a few roundings times the sums over points)."""
+    import torch
+    from paper_2101_12597_gb300.etdm import ETDM
+    d = synth.crystal(cells=(2, 2, 12), spacing_ang=2.6, Z=2.0, rcut_ang=3.0, kT_ev=0.5, a_sigma=0.05,
+                      seed=12, exps=exps, grid=(14, 14, 84), kmesh=2)
+    bo = BlochOracle(d)
+    C0 = bo.lowdin_reference()
+    f = np.zeros(bo.M)
+    f[:bo.M // 2:2] = 1.0  # an orbital of each atom of the first half
+    f *= bo.N / f.sum()
+    occ = [2.0 * w * f for w in bo.kw]
+    bo.reference_k()
+    bo.set_reference(C0, occ)
+    s = ETDM(d)
+    s.set_reference(np.array(C0), np.array(occ))
+    a = np.zeros(bo.nk * bo.nvar)
+    E, g = s.energy_grad(torch.tensor(a, dtype=torch.float64, device="cuda"))
+    torch.cuda.synchronize()
+    s.check()
+    E_ref, g_ref, ex = bo.energy_grad(a, want=True)
+    D = s.get_array("D_k").reshape(bo.nk, bo.M, bo.M)
+    H = s.get_array("H_k").reshape(bo.nk, bo.M, bo.M)
+    ref, mag, dH, big = np.zeros(bo.G), np.zeros(bo.G), 0.0, 0.0
+    for k in range(bo.nk):
+        X = bo.Xk(k)
+        ref += ((X @ D[k]) * X.conj()).sum(1).real
+        mag += ((np.abs(X) @ np.abs(D[k])) * np.abs(X)).sum(1)
+        dH = max(dH, np.abs(H[k] - ex["k"][k]["H"]).max())
+        big = max(big, np.abs(ex["k"][k]["H"]).max())
+    err = (np.abs(s.get_array("rho").reshape(-1) - ref) / mag).max()
+    print(f"{exps}: rho {err:.1e}, H {dH:.1e} of {big:.1e}, smallest rho {mag.min():.1e}")
+    assert err <= TOL and dH <= 64 * 2.0 ** -53 * big
+    assert abs(float(E.item()) - E_ref) < 1e-9
+    s.close()
