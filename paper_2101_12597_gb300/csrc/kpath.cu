@@ -46,6 +46,19 @@ cudaError_t prod_k(etdm_handle *h, const double2 *A, int opa, const double2 *B, 
   return zgemm_sq(A, opa, B, opb, C, h->M, h->nk, s, alpha, beta);
 }
 
+// O = C0 U (U is overwritten).  On the tensor cores as C0 + C0 (U - I): their
+// error is relative to the largest elements of a row and of a column, and near
+// the reference, or where A(k) leaves orbitals alone, those of U - I are small.
+void orbitals_k(etdm_handle *h, double2 *U, double2 *O, cudaStream_t s) {
+  const bool oz = h->oz.n == h->M;
+  if (oz) {
+    CUDA_TRY(k_less_identity(U, h->nk, h->M, s));
+    CUDA_TRY(cudaMemcpyAsync(O, h->d_kC0, (size_t)h->nk * h->M * h->M * 16, cudaMemcpyDeviceToDevice, s));
+    h->launches += 1;
+  }
+  CUDA_TRY(prod_k(h, h->d_kC0, 0, U, 0, O, s, 1.0, oz ? 1.0 : 0.0));
+}
+
 }  // namespace
 
 void init_kpoints(etdm_handle *h, const etdm_system *sys) {
@@ -242,7 +255,7 @@ void refresh_reference_k(etdm_handle *h, cudaStream_t s) {
 void reference_update_k(etdm_handle *h, double *a, cudaStream_t s) {
   const int M = h->M, nk = h->nk;
   expm_ss_k(h, a, h->d_kW, s);
-  CUDA_TRY(prod_k(h, h->d_kC0, 0, h->d_kW, 0, h->d_kX1, s));
+  orbitals_k(h, h->d_kW, h->d_kX1, s);
   CUDA_TRY(cudaMemcpyAsync(h->d_kC0, h->d_kX1, (size_t)nk * M * M * 16, cudaMemcpyDeviceToDevice, s));
   CUDA_TRY(cudaMemsetAsync(a, 0, h->nvar * 8, s));
   refresh_reference_k(h, s);
@@ -289,14 +302,19 @@ void evaluate_k(etdm_handle *h, const double *a, double *E, double *g, cudaStrea
   }
   StageTimer tf(h, s, ETDM_STAGE_DENSE_FWD);
   if (ss) {
-    CUDA_TRY(prod_k(h, h->d_kC0, 0, h->d_kW, 0, h->d_kO, s));    // O = C0 U
+    orbitals_k(h, h->d_kW, h->d_kO, s);
   } else {
     CUDA_TRY(k_colscale(h->d_kW, h->d_komega, h->d_kX1, nk, M, 2, h->d_flags, s));
     CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kW, 1, h->d_kX2, s));    // U
-    CUDA_TRY(prod_k(h, h->d_kC0, 0, h->d_kX2, 0, h->d_kO, s));    // O = C0 U
+    orbitals_k(h, h->d_kX2, h->d_kO, s);
   }
-  CUDA_TRY(k_colscale(h->d_kO, h->d_kf, h->d_kX1, nk, M, 0, h->d_flags, s));
-  CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kO, 1, h->d_kD, s));     // D = O f O^dagger
+  if (h->oz.n == M) {  // D = O f O^dagger
+    CUDA_TRY(k_occ_factors(h->d_kO, h->d_kf, h->d_kX1, h->d_kX2, nk, M, s));
+    CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kX2, 1, h->d_kD, s));
+  } else {
+    CUDA_TRY(k_colscale(h->d_kO, h->d_kf, h->d_kX1, nk, M, 0, h->d_flags, s));
+    CUDA_TRY(prod_k(h, h->d_kX1, 0, h->d_kO, 1, h->d_kD, s));
+  }
   CUDA_TRY(k_dr(G, h->d_kD, h->d_kDR, s));
   tf.done();
   // density, potential, energy

@@ -72,6 +72,10 @@ cudaError_t k_fro2(const double2 *X, long n, double *part, cudaStream_t s);
 // X = Y diag(s): mode 0 s = x, mode 1 s = x^(-1/2), mode 2 s = exp(-i x)
 cudaError_t k_colscale(const double2 *Y, const double *x, double2 *X, int nk, int M, int mode,
                        int *flags, cudaStream_t s);
+// X1 X2^dagger = O f O^dagger in two factors of like size
+cudaError_t k_occ_factors(const double2 *O, const double *f, double2 *X1, double2 *X2, int nk, int M,
+                          cudaStream_t s);
+cudaError_t k_less_identity(double2 *U, int nk, int M, cudaStream_t s);
 cudaError_t k_hermitize(double2 *X, int nk, int M, cudaStream_t s);
 cudaError_t k_phases(const KGeom &G, double2 *phase, cudaStream_t s);  // fills G.phase's table (set-up)
 cudaError_t k_dr(const KGeom &G, const double2 *D, double *DR, cudaStream_t s);

@@ -21,6 +21,12 @@
 //   - the read-out adds the eight exact integers of a chunk into two 64-bit
 //     integers per output (orders 0-3 and 4-7), and one FP64 multiply-add at
 //     the end gives the result, rounded once.
+// The error is relative to the largest elements of the row and the column, not to
+// the terms of the sum as in FP64: K 2^-61 |A_i| |B_j| at most.  Factors that are
+// products themselves carry 2^-53 of those norms already; where elements far
+// below them matter and may be exact (rho^(1/3) of orbitals' tails) the caller
+// makes the factors of like size: O = C0 + C0 (U - I), and O f O^dagger in two
+// factors O f^(1/2).
 // A complex matrix product is one real product with K' = 2k: A' rows are the
 // (re, im) pairs as stored, B' has two rows per column j of B, (re, -im) for
 // the real and (im, re) for the imaginary part of C_ij, which come out
