@@ -266,12 +266,35 @@ void init_batch(etdm_handle *h, const etdm_system *sys, int n_sys, const etdm_op
   h->lbfgs_m = o.lbfgs_m;
   h->gamma = o.gamma;
   h->beta0 = o.beta0;
+  // The FP64 members' tables are optional: they are given back when a later
+  // member has no room for what it cannot do without, and not taken again
+  bool tables = true;
+  auto give_back = [h] {
+    bool any = false;
+    CUDA_TRY(cudaDeviceSynchronize());
+    for (etdm_handle *m : h->members)
+      if (m->ox.n_tiles) {
+        dfree(m, m->ox.x);
+        m->ox = OxGrid{};
+        any = true;
+      }
+    return any;
+  };
   for (int i = 0; i < n_sys; ++i) {
     etdm_handle *m = new etdm_handle();
+    m->tables = tables;
     h->members.push_back(m);
     try {
       init_system(m, &sys[i], &o);
     } catch (Fail &f) {
+      if (f.code == ETDM_ERR_OOM && tables && give_back()) {
+        tables = false;
+        h->members.pop_back();
+        release_handle(m);
+        delete m;
+        --i;
+        continue;
+      }
       f.msg = "system " + std::to_string(i) + ": " + f.msg;
       throw;
     }

@@ -385,6 +385,7 @@ void etdm::build_vgroups(etdm_handle *h, int vg_max, cudaStream_t s) {
 }
 
 void etdm::setup_ox(etdm_handle *h, bool images, cudaStream_t s) {
+  if (!h->tables) return;
   int T = 0, max_list = 0, *d_ptr = nullptr, *d_keys = nullptr;
   long n = 0;
   const GridGeom geom = make_geom(h, 4, 4, 8, &T);

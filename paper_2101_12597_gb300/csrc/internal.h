@@ -334,6 +334,7 @@ struct etdm_handle {
   void *d_kwork = nullptr;      // eigensolver workspace
   etdm::OzWork oz{};            // tensor-core products (large M)
   etdm::OxGrid ox{};            // FP64 grid passes on the tensor cores
+  bool tables = true;           // set-up may take memory for them
   bool kref_set = false;        // reference given by etdm_set_reference
   int kexpm = 0;                // ETDM_EXPM_EIG (Eq. 35, Eq. 39) or ETDM_EXPM_SS (Eq. 38, Eq. 42)
   int tri_method = 1;           // tridiagonal eigenpairs of iA(k): 1 bisection + inverse iteration, 0 QL

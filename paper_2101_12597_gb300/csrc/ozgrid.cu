@@ -755,7 +755,7 @@ void ox_setup(etdm_handle *h, const GridGeom &geom, int n_tiles, const std::vect
     p += (n + 255) & ~(size_t)255;
     return q;
   };
-  o.x = (long long *)take((size_t)ne * kOxP * 8);
+  o.x = (long long *)take((size_t)ne * kOxP * 8);  // (the allocation's address)
   o.xt = (long long *)take((size_t)ne * kOxP * 8);
   o.vt = (long long *)take((size_t)n_tiles * kOxP * 8);
   o.dfix = (long long *)take((size_t)mats * MM * 8);

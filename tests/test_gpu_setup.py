@@ -67,3 +67,40 @@ def test_setup_without_room_for_the_tables(path):
     print(f"{path}: {takes >> 20} MB, launches {n0} -> {n1}, dE={abs(E1 - E0):.1e} dg={dg:.1e}")
     assert n1 < n0  # the passes on tables take more launches
     assert abs(E1 - E0) < 1e-9 and dg <= 1e-9
+
+
+def test_batch_without_room_for_every_table():
+    """An FP64 batch whose members fit without their tables: those of the first
+    members are given back when a later one has no room."""
+    import torch
+    from paper_2101_12597_gb300.etdm import ETDMBatch
+    systems = [synth.water_box(lattice=(3, 2, 2), box_ang=7.4, grid=(56, 56, 56), rcut_ang=3.5, seed=i)
+               for i in range(8)]
+    a = torch.tensor(np.concatenate([d["a0"].ravel() for d in systems]), device="cuda")
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    ETDMBatch(systems[:1], precision="fp64").close()
+    before = free()
+    b = ETDMBatch(systems, precision="fp64")
+    takes = before - free()
+    E0, g0 = (x.clone() for x in b.energy_grad(a))
+    torch.cuda.synchronize()
+    b.close()
+    # room for three members with their tables and part of a fourth's memory
+    leave = int(3.2 * takes / len(systems))
+    fill = torch.empty(free() - leave, dtype=torch.uint8, device="cuda")
+    try:
+        b = ETDMBatch(systems, precision="fp64")
+        E1, g1 = (x.clone() for x in b.energy_grad(a))
+        torch.cuda.synchronize()
+        b.close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    print(f"{takes >> 20} MB, {leave >> 20} left: dE={(E1 - E0).abs().max().item():.1e}")
+    assert (E1 - E0).abs().max().item() < 1e-9
+    assert (g1 - g0).abs().max().item() <= 1e-9 * g0.abs().max().item()
