@@ -215,7 +215,8 @@ __device__ __forceinline__ int ox_dexp(double d) { return (exp_field(d) - 1021) 
 constexpr int kOxBad = (kOzBad - 1021) >> 1;
 
 // D_ab 2^-(e_a + e_b) (one bit in reserve for rounding), the exponents and the
-// tiles' largest ones (kOxBad: no number), the points' shifts pmin; diag: the offset 0 of DR (its diagonal bounds every offset)
+// tiles' largest ones (kOxBad: no number), the points' shifts pmin; diag: the
+// offset 0 of DR (its diagonal bounds every offset)
 __global__ void __launch_bounds__(256) ox_dfix_kernel(const double *D, long n, const double *diag, int M,
                                                       int shift, int n_tiles, const int *ptr, const int *id,
                                                       const uint32_t *kx, long long *dst, int *ee, int *ct,
